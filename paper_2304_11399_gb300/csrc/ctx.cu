@@ -62,6 +62,8 @@ tt::EvalArgs tt_ctx::eval_args(const float* theta, int P, float* S) const {
   a.split = split ? 1 : 0;
   a.split_blocks = 1;
   a.n_sm = n_sm;
+  a.n_groups = n_groups;
+  a.mean_ap = n_dom > 0 ? float(sum_N / n_dom) : 0.f;
   a.split_part = split_part;
   a.split_part_d = split_part_d;
   a.split_ticket = split_ticket;

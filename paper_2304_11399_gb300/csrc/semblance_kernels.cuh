@@ -134,7 +134,10 @@ struct Pos {
   float q;     // p0 + A' dm (for the gradient)
 };
 
-template <int OP, bool MOVEOUT>
+// FLOOR_FP32: the direct form's floor of 0 <= u < 2^23 by adding 2^23 rounded
+// toward zero -- FP32-pipe work with the same result, for kernels that do
+// little else per position; truncf and the conversion take the slow unit twice.
+template <int OP, bool MOVEOUT, bool FLOOR_FP32 = false>
 __device__ __forceinline__ Pos locate(const Lane& L, float4 t4) {
   Pos P;
   if (!MOVEOUT) {
@@ -150,10 +153,17 @@ __device__ __forceinline__ Pos locate(const Lane& L, float4 t4) {
       U = fmaf(P.q, P.q, fo_quad(L, t4));
     }
     P.u = fminf(sqrt_approx(U), L.umax);
-    const float fl = truncf(P.u);
-    P.f = __fsub_rn(P.u, fl);
+    if (FLOOR_FP32) {
+      const float big = __fadd_rz(P.u, 8388608.f);
+      const float fl = __fsub_rn(big, 8388608.f);
+      P.f = __fsub_rn(P.u, fl);
+      P.j = int(__float_as_uint(big) - 0x4b000000u);
+    } else {
+      const float fl = truncf(P.u);
+      P.f = __fsub_rn(P.u, fl);
+      P.j = int(fl);
+    }
     P.g = __fsub_rn(1.f, P.f);
-    P.j = int(fl);
     return P;
   }
   float V, x;
@@ -670,31 +680,79 @@ __global__ void __launch_bounds__(kBlock) k_semblance_grad(const EvalArgs a) {
 
 using KFn = void (*)(const EvalArgs);
 
-// Stacked output: one warp per domain (P = 1, theta [n_dom][D]); lane l sums
-// the centre amplitudes of aperture entries e0 + l, e0 + l + 32, ... in order,
-// the 32 lane sums meet in a butterfly, and the mean is one FP32 division.
-// Positions are those of the semblance window's centre sample (same clamp:
-// T < 0 or past the record reads the zero padding).
+// Stacked output (P = 1, theta [n_dom][D]): 32 strided sums of the centre
+// amplitudes -- sum l takes aperture entries e0 + l, e0 + l + 32, ... in order
+// -- added in a butterfly (sums 16 apart, then 8, ...), and the mean is one
+// FP32 division. Positions are those of the semblance window's centre sample
+// (same clamp: T < 0 or past the record reads the zero padding). Two forms
+// with the same operations, so the same bits.
+template <int OP, typename T, bool MV>
+__device__ __forceinline__ float centre(const EvalArgs& a, const Lane& L, int e, float s) {
+  const float4 t4 = __ldg(a.ap_tab + e);
+  const Pos P = locate<OP, MV, true>(L, t4);
+  const T* x = static_cast<const T*>(a.traces) + (__float_as_uint(t4.w) + P.j);
+  return __fadd_rn(s, fmaf(P.f, ld_sample<T>(x + 1), __fmul_rn(P.g, ld_sample<T>(x))));
+}
+
+// Domains with apertures of their own: one warp per domain, lane l taking sum l.
 template <int OP, typename T, bool MV>
 __global__ void __launch_bounds__(256) k_stack(const EvalArgs a, float* __restrict__ out) {
   const long long d = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   Lane L;
   if (!lane_setup<OP>(a, d, L)) return;  // warp-uniform: the whole warp leaves
-  const T* __restrict__ tr = static_cast<const T*>(a.traces);
   float s = 0.f;
-  for (int e = L.e0 + lane; e < L.e1; e += 32) {
-    const float4 t4 = __ldg(a.ap_tab + e);
-    const Pos P = locate<OP, MV>(L, t4);
-    const T* x = tr + (__float_as_uint(t4.w) + P.j);
-    s = __fadd_rn(s, fmaf(P.f, ld_sample<T>(x + 1), __fmul_rn(P.g, ld_sample<T>(x))));
-  }
+  for (int e = L.e0 + lane; e < L.e1; e += 32) s = centre<OP, T, MV>(a, L, e, s);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
   if (lane == 0) {
     const int N = L.e1 - L.e0;
     out[L.d] = N > 0 ? __fdiv_rn(s, float(N)) : 0.f;
   }
+}
+
+// Domains that share apertures (consecutive t0 of one midpoint): one lane per
+// domain, so that a warp walks the same entries and reads one trace row at 32
+// neighbouring positions (a line or two a request, against 32 lines where a
+// warp spreads over 32 rows). 32 / R warps share 32 domains, each holding R of
+// their sums in registers; the sums meet in shared memory.
+template <int OP, typename T, bool MV, int R>
+__global__ void __launch_bounds__(R == 1 ? 1024 : 256) k_stack_rows(const EvalArgs a,
+                                                                     float* __restrict__ out) {
+  constexpr int NW = R == 1 ? 32 : 8;  // warps per block
+  constexpr int per = 32 / R;          // warps per 32 domains
+  __shared__ float sums[NW / per][32][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int g = w / per, l0 = (w - g * per) * R;
+  const long long d = ((long long)blockIdx.x * (NW / per) + g) * 32 + lane;
+  Lane L;
+  const bool valid = lane_setup<OP>(a, d, L);
+  float s[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) s[r] = 0.f;
+  if (valid) {
+    int e = L.e0 + l0;
+    for (; e + R <= L.e1; e += 32) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) s[r] = centre<OP, T, MV>(a, L, e + r, s[r]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (e + r < L.e1) s[r] = centre<OP, T, MV>(a, L, e + r, s[r]);
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) sums[g][lane][l0 + r] = s[r];
+  __syncthreads();
+  if (l0 != 0 || !valid) return;
+  float t[32];
+#pragma unroll
+  for (int l = 0; l < 32; ++l) t[l] = sums[g][lane][l];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int l = 0; l < o; ++l) t[l] = __fadd_rn(t[l], t[l + o]);
+  const int N = L.e1 - L.e0;
+  out[L.d] = N > 0 ? __fdiv_rn(t[0], float(N)) : 0.f;
 }
 
 // Member order of one population for the evaluation that follows: one warp
@@ -750,7 +808,9 @@ OFn pick_order(bool mv) {
 }
 
 using SFn = void (*)(const EvalArgs, float*);
-enum KernelKind { kKindPacked = 0, kKindScalar = 1, kKindSplit = 2, kKindGrad = 3 };
+enum KernelKind {
+  kKindPacked = 0, kKindScalar = 1, kKindSplit = 2, kKindGrad = 3
+};
 
 template <int OP, int W, typename T, bool MV>
 KFn pick_kind(int kind) {
@@ -788,11 +848,26 @@ KFn pick_kernel(int kind, int storage, int W, bool mv) {
   return bf ? pick_w<OP, __nv_bfloat16, false>(kind, W) : pick_w<OP, float, false>(kind, W);
 }
 
+// The stack kernel of operator OP: rows = 0 the warp-per-domain form, else the
+// lane-per-domain form with that many sums per warp.
+template <int OP, typename T, bool MV>
+SFn pick_stack_rows(int rows) {
+  switch (rows) {
+    case 0: return k_stack<OP, T, MV>;
+    case 1: return k_stack_rows<OP, T, MV, 1>;
+    case 8: return k_stack_rows<OP, T, MV, 8>;
+  }
+  return nullptr;
+}
+
 template <int OP>
-SFn pick_stack(int storage, bool mv) {
+SFn pick_stack(int storage, bool mv, int rows) {
   const bool bf = storage == TT_STORE_BF16;
-  if (mv) return bf ? k_stack<OP, __nv_bfloat16, true> : k_stack<OP, float, true>;
-  return bf ? k_stack<OP, __nv_bfloat16, false> : k_stack<OP, float, false>;
+  if (mv)
+    return bf ? pick_stack_rows<OP, __nv_bfloat16, true>(rows)
+              : pick_stack_rows<OP, float, true>(rows);
+  return bf ? pick_stack_rows<OP, __nv_bfloat16, false>(rows)
+            : pick_stack_rows<OP, float, false>(rows);
 }
 
 }  // namespace sk

@@ -77,6 +77,8 @@ struct EvalArgs {
   double* split_part_d;     // [split_part_sets][64] block partial FP64 energies
   unsigned* split_ticket;   // [split_tickets] arrivals per unit, zero between launches
   unsigned long long* queue;  // persistent mode: work-unit counter, zero at launch
+  int n_groups;             // aperture groups of the context
+  float mean_ap;            // mean aperture size over the context's domains
 };
 
 cudaError_t launch_semblance(const EvalArgs& a, cudaStream_t s);

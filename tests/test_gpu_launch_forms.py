@@ -1,0 +1,58 @@
+"""Forms of a launch that compute the same thing, compared at the sizes where
+the forms change or a tile is ragged."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2304_11399_gb300 as tt
+from gpu_util import dev, random_theta, synth, to_dev, configs
+
+pytestmark = pytest.mark.gpu
+
+BOUNDS = {1: (configs.CRS_LO, configs.CRS_HI), 2: (configs.FO_LO, configs.FO_HI)}
+
+
+def _problem(n_dom, sizes, n_tr, ns, op=1, w=5, own_groups=False, seed=0):
+    """n_dom domains over len(sizes) groups of the given aperture sizes;
+    own_groups: the same domains, each with a group (a copy) of its own."""
+    rng = np.random.default_rng(seed)
+    lists = [rng.integers(0, n_tr, n).astype(np.int32) for n in sizes]
+    grp = np.sort(rng.integers(0, len(sizes), n_dom))
+    it0 = rng.integers(0, ns, n_dom).astype(np.int32)
+    m0 = rng.uniform(0, 100, len(sizes)).astype(np.float32)
+    if own_groups:
+        lists, m0, grp = [lists[g] for g in grp], m0[grp], np.arange(n_dom)
+    G = len(lists)
+    return synth.Problem(op=op, half_window=w, group_m0=m0,
+                         group_dt=np.full(G, 0.004, np.float32),
+                         ap_ptr=np.concatenate([[0], np.cumsum([x.size for x in lists])]).astype(np.int32),
+                         ap_idx=np.concatenate(lists + [np.zeros(0, np.int32)]).astype(np.int32),
+                         dom_it0=it0, dom_group=grp.astype(np.int32),
+                         group_h0=np.full(G, 400.0, np.float32) if op == 2 else None)
+
+
+def _line(n_tr, ns, seed=1):
+    rng = np.random.default_rng(seed)
+    return (rng.standard_normal((n_tr, ns)).astype(np.float32),
+            rng.uniform(0, 100, n_tr).astype(np.float32),
+            rng.uniform(0, 900, n_tr).astype(np.float32))
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+@pytest.mark.parametrize("ns", [300, 2200])  # direct and moveout positions
+@pytest.mark.parametrize("n_dom,sizes", [
+    (31, (1,)), (32, (31, 33)), (33, (0, 32)), (700, (64, 7, 100)), (80001, (40,))])
+def test_stack_lane_and_warp_per_domain_bit_identical(n_dom, sizes, ns, storage):
+    """Lane-per-domain form (domains that share apertures; one sum per warp,
+    and eight from about 78,000 domains on) against the warp-per-domain form
+    (the same domains with apertures of their own)."""
+    x, mid, off = _line(50, ns)
+    th = to_dev(random_theta(n_dom, 1, *BOUNDS[1], 3)[:, 0])
+    outs = []
+    for own in (False, True):
+        ctx = tt.tt_ctx_create(x, mid, off, _problem(n_dom, sizes, 50, ns, own_groups=own), None,
+                               storage=storage, device=dev())
+        outs.append(tt.tt_stack(ctx, th))
+        ctx.close()
+    assert torch.equal(outs[0], outs[1])
