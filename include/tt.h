@@ -23,8 +23,7 @@
  *    asynchronous launch. tt_last_error() gives a message.
  *  - A context may be used from one host thread at a time; calls on
  *    different streams that share a context's scratch (tt_search,
- *    tt_ens_search, tt_neighbor_exchange, tt_polish, split evaluations --
- *    see TT_OPT_SPLIT) must not overlap.
+ *    tt_ens_search, tt_neighbor_exchange, tt_polish) must not overlap.
  *
  * Notation (the paper's): a domain is one zero-offset sample (m0, it0),
  * t0 = it0 dt (Sec. 2.1, "index-vector point (t, tr)"); its aperture is the
@@ -333,18 +332,13 @@ tt_status tt_ctx_probe_l1(tt_ctx* ctx, int32_t iters, double* bytes, void* strea
  *                 n_sm x 32 x 64 (domain, vector) pairs, n_sm the device's
  *                 multiprocessor count (TT_OPT_SPLIT_MAX_PAIRS reads the
  *                 figure) -- too few to fill the GPU at one warp per 64
- *                 pairs -- runs a kernel in which
- *                 the S warps of a block (8, 16 or 32, more for smaller
- *                 launches) share 64 pairs, each warp summing a contiguous
- *                 slice of every pair's aperture, the partial sums added in
- *                 slice order; every variant then launches that kernel, so S
+ *                 pairs -- cuts every pair's aperture into 8 B contiguous
+ *                 slices shared by the warps of one or more blocks (B = 1, 2,
+ *                 7 or 9, more for smaller launches), the partial sums added in
+ *                 slice order; every variant then sums alike, so S
  *                 still does not depend on TT_OPT_KERNEL / TT_OPT_BLOCK, but
  *                 its rounding differs from the unsplit kernels' (all stay
- *                 within 1e-5 of the exact semblance). The smallest launches
- *                 also spread a unit over up to 9 blocks that combine their
- *                 sums through the context's scratch, so split evaluations on
- *                 one context must not overlap on the GPU (one stream, or
- *                 events between streams). 0: never split.
+ *                 within 1e-5 of the exact semblance). 0: never split.
  *  TT_OPT_MEMBER_ORDER  1: before each generation's evaluation inside
  *                 tt_search / tt_search_slab (NP <= 256), the members of
  *                 every domain are put in the order of their window position

@@ -64,9 +64,6 @@ tt::EvalArgs tt_ctx::eval_args(const float* theta, int P, float* S) const {
   a.n_sm = n_sm;
   a.n_groups = n_groups;
   a.mean_ap = n_dom > 0 ? float(sum_N / n_dom) : 0.f;
-  a.split_part = split_part;
-  a.split_part_d = split_part_d;
-  a.split_ticket = split_ticket;
   a.queue = queue;
   return a;
 }
@@ -348,8 +345,7 @@ void free_ctx(tt_ctx* c) {
                   c->dom_it0, c->dom_group, c->bounds, c->pop, c->fit, c->trial[0],
                   c->trial[1], c->tfit[0], c->tfit[1], c->snap, c->imports, c->slots,
                   c->best_idx, c->pol_th, c->pol_g, c->pol_S, c->pol_bth, c->pol_bS, c->d_err,
-                  c->queue, c->split_part, c->split_part_d, c->split_ticket, c->split_part2,
-                  c->split_part_d2, c->split_ticket2, c->out_th,
+                  c->queue, c->probe, c->out_th,
                   c->out_S, c->jade_mu, c->jade_arc, c->jade_F,
                   c->jade_CR, c->jade_na};
   for (void* p : ptrs)
@@ -608,18 +604,7 @@ extern "C" tt_status tt_ctx_create(tt_ctx** out, const tt_gathers* ga, const tt_
     }
   }
   TRY(dalloc(&c->queue, 1), "alloc queue");
-  TRY(dalloc(&c->split_part, size_t(tt::split_part_sets(c->n_sm)) * 64 * tt::kSplitPartStride),
-      "alloc split scratch");
-  TRY(dalloc(&c->split_part_d, size_t(tt::split_part_sets(c->n_sm)) * 64), "alloc split scratch");
-  TRY(dalloc(&c->split_ticket, size_t(tt::split_tickets(c->n_sm))), "alloc split tickets");
-  TRY(cudaMemsetAsync(c->split_ticket, 0, size_t(tt::split_tickets(c->n_sm)) * sizeof(unsigned), s),
-      "clear split tickets");
-  TRY(dalloc(&c->split_part2, size_t(tt::split_part_sets(c->n_sm)) * 64 * tt::kSplitPartStride),
-      "alloc split scratch");
-  TRY(dalloc(&c->split_part_d2, size_t(tt::split_part_sets(c->n_sm)) * 64), "alloc split scratch");
-  TRY(dalloc(&c->split_ticket2, size_t(tt::split_tickets(c->n_sm))), "alloc split tickets");
-  TRY(cudaMemsetAsync(c->split_ticket2, 0, size_t(tt::split_tickets(c->n_sm)) * sizeof(unsigned), s),
-      "clear split tickets");
+  TRY(dalloc(&c->probe, tt::kProbeFloats), "alloc probe window");
   {
     size_t nd = size_t(c->n_dom), Dz = size_t(D);
     TRY(dalloc(&c->out_th, nd * Dz), "alloc search output");

@@ -216,8 +216,7 @@ tt_status ens_body(tt_ctx* c, const tt_ens_cfg& e, float* bth, float* bS, cudaSt
   // The interpolated samples of a step (interpolate, evaluate, keep) only
   // touch that trace's skipped samples, which the next steps of the stage do
   // not read; they run on the side stream, overlapping the next step, with
-  // their maps and buffers double-buffered by step parity and their own
-  // split scratch. A step waits for the side work of the step two before it
+  // their maps and buffers double-buffered by step parity. A step waits for the side work of the step two before it
   // (which used the same buffers); every stage ends with a join.
   if (!c->side_stream) {
     cudaError_t r = cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking);
@@ -333,9 +332,6 @@ tt_status ens_body(tt_ctx* c, const tt_ens_cfg& e, float* bth, float* bS, cudaSt
         tt::EvalArgs ei = c->eval_args(th_skp, 1, S_skp);
         ei.n_dom = n_skp_loc;
         ei.dom_map = map_skp;
-        ei.split_part = c->split_part2;
-        ei.split_part_d = c->split_part_d2;
-        ei.split_ticket = c->split_ticket2;
         STEP(c->semblance(ei, s2, false), "ens evaluate interpolated");
         calls += (unsigned long long)active * g.n_skp;
         k_ens_keep<<<blocks(n_skp_loc), 256, 0, s2>>>(n_skp_loc, D, map_skp, th_skp, S_skp, bth,

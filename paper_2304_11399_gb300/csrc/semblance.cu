@@ -31,6 +31,60 @@ KFn pick(int kind, const EvalArgs& a, bool mv) {
   return nullptr;
 }
 
+// A block's shared memory above 48 KB, the kernel's own arrays included, has
+// to be asked for.
+template <typename Fn>
+cudaError_t allow_smem(Fn fn, size_t bytes) {
+  if (bytes <= 40 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+}
+
+// Sums of eight slices per pair of a split launch (see semblance_kernels.cuh).
+int split_blocks(long long units, int n_sm) {
+  return units * 2 <= n_sm                              ? kSplitTinyBlocks
+         : units <= (long long)n_sm * kSplitSmallPerSm ? kSplitSmallBlocks
+         : units < (long long)n_sm * kSplitMultiPerSm  ? 2
+                                                       : 1;
+}
+
+cudaError_t launch_split(EvalArgs& a, long long units, bool mv, cudaStream_t s) {
+  const bool bf = a.storage == TT_STORE_BF16;
+  const int B = split_blocks(units, a.n_sm);
+  a.split_blocks = B;
+  // 7 warps a unit instead of 56 while they are not walked for longer than the
+  // 56 take to come and go: 48 traces 118 / 258 units 8.7 / 10.4 us against
+  // 10.5 / 18.5 us, 144 traces 258 units 18.6 against 22.8 us; 336 traces 118 /
+  // 258 units 20.7 / 34.9 us against 16.7 / 31.1 us
+  if (B == kSplitSmallBlocks && a.mean_ap <= 0.6f * float(units)) {
+    const KFn fn = pick(sk::kKindShort, a, mv);
+    if (!fn) return cudaErrorInvalidValue;
+    const size_t smem = sk::short_smem_bytes(kSplitSmallBlocks, a.W, bf);
+    const cudaError_t e = allow_smem(fn, smem);
+    if (e != cudaSuccess) return e;
+    fn<<<unsigned(units), 32 * kSplitSmallBlocks, smem, s>>>(a);
+    return cudaGetLastError();
+  }
+  const KFn fn = pick(sk::kKindSplit, a, mv);
+  if (!fn) return cudaErrorInvalidValue;
+  const size_t smem = sk::split_smem_bytes(B, a.W, bf);
+  cudaError_t e = allow_smem(fn, smem);
+  if (e == cudaSuccess && B > 8)  // more blocks than every device has to offer
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = unsigned(B);
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(units * B));
+  cfg.blockDim = dim3(32 * sk::kSplitWarps);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, a);
+}
+
 cudaError_t launch(const EvalArgs& a, cudaStream_t s, bool grad) {
   const long long n = (long long)a.n_dom * a.P;
   if (n == 0) return cudaSuccess;
@@ -44,28 +98,8 @@ cudaError_t launch(const EvalArgs& a, cudaStream_t s, bool grad) {
     fn = pick(sk::kKindGrad, a, mv);
     blocks = (n + block - 1) / block;
   } else if (a.split && (n + 63) / 64 < (long long)a.n_sm * kSplitUnitsPerSm) {
-    // too few units to fill the GPU: each unit's aperture split over the
-    // warps of B blocks, (S, B) by launch size only
-    fn = pick(sk::kKindSplit, a, mv);
-    if (!fn) return cudaErrorInvalidValue;
-    const long long units = (n + 63) / 64;
-    int S = sk::split_warps(units, a.n_sm);
-    b.split_blocks = 1;
-    if (a.split_part && a.split_ticket) {
-      if (units <= (long long)a.n_sm * kSplitSmallPerSm) {
-        S = sk::kSplitMultiWarps;
-        b.split_blocks = units * 2 <= a.n_sm ? kSplitTinyBlocks : kSplitSmallBlocks;
-      } else if (units < (long long)a.n_sm * kSplitMultiPerSm) {
-        S = 8;
-        b.split_blocks = 2;
-      }
-    }
-    const size_t smem = sk::split_smem_bytes(S, a.W);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(sk::split_smem_bytes(sk::kSplitMaxWarps, a.W)));
-    if (e != cudaSuccess) return e;
-    fn<<<unsigned(units * b.split_blocks), 32 * S, smem, s>>>(b);
-    return cudaGetLastError();
+    // too few units to fill the GPU: each unit's aperture split over warps
+    return launch_split(b, (n + 63) / 64, mv, s);
   } else if (a.kernel == TT_KERNEL_SCALAR) {
     fn = pick(sk::kKindScalar, a, mv);
     blocks = (n + block - 1) / block;
@@ -217,9 +251,9 @@ extern "C" tt_status tt_semblance_grad(tt_ctx* ctx, const float* theta, int32_t 
 extern "C" tt_status tt_ctx_probe_l1(tt_ctx* ctx, int32_t iters, double* bytes, void* stream) {
   if (!ctx) return tt_fail(nullptr, TT_ERR_INVALID_ARG, "ctx is NULL");
   if (iters < 1 || !bytes) return tt_fail(ctx, TT_ERR_INVALID_ARG, "iters < 1 or bytes is NULL");
-  // the window and the sink live in the context's split scratch (no allocation)
+  // the window and the sink live in the context (no allocation)
   return tt_cuda_check(ctx,
-                       ctx->counted(tt::launch_l1_probe(ctx->split_part, ctx->split_part + 8192,
+                       ctx->counted(tt::launch_l1_probe(ctx->probe, ctx->probe + 8192,
                                                         ctx->n_sm, iters, bytes,
                                                         static_cast<cudaStream_t>(stream))),
                        "L1 probe launch");

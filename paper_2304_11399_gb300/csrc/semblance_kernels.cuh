@@ -37,11 +37,25 @@
 // may fuse), so they agree bit for bit.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include "tt_internal.cuh"
 
 namespace tt {
 namespace sk {
 
+
+// The two halves of a cluster barrier: work between them overlaps the other
+// blocks' arrival. The relaxed arrival orders no memory (no fence to wait for).
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 
 __device__ __forceinline__ float sqrt_approx(float x) {
   float y;
@@ -77,12 +91,20 @@ struct Lane {
   float umax;          // direct: u is clamped to ns + w
 };
 
+// Domain of pair q = d P + p. A 64-bit division costs about a hundred
+// instructions a lane, which the short-lived warps of the split kernels feel.
+__device__ __forceinline__ int dom_of(long long q, int P) {
+  if (P == 1) return int(q);
+  if (q <= 0x7fffffffll) return int(unsigned(q) / unsigned(P));
+  return int(q / P);
+}
+
 // L.d is the local domain (indexing theta and S); its geometry comes from the
 // global domain dom_map[L.d] when a map is given (a subset evaluation).
-template <int OP>
+template <int OP, bool DIV32 = false>
 __device__ __forceinline__ bool lane_setup(const EvalArgs& a, long long q, Lane& L) {
   if (q >= (long long)a.n_dom * a.P) return false;
-  L.d = int(q / a.P);
+  L.d = DIV32 ? dom_of(q, a.P) : int(q / a.P);
   const int gd = a.dom_map ? a.dom_map[L.d] : L.d;
   if (gd < 0) return false;
   const int g = a.dom_group[gd];
@@ -402,69 +424,97 @@ __device__ __forceinline__ void eval_unit(const EvalArgs& a, long long unit, int
   store_S(a, q1, L1.d, normalise<T>(Q.y, N, E.y, Ed1));
 }
 
-// K1 for small launches (few 64-pair units): B blocks of S warps share one
-// unit, warp w of block b walking slice b S + w of the B S contiguous slices
-// of every pair's aperture. Within a block the slices' partial sums meet in
-// shared memory and are added in slice order; with B > 1 each block writes
-// its sums to global scratch and the last block of the unit to arrive (an
-// atomic ticket, no waiting) adds the B block sums in block order. (S, B)
-// is (8, 9) up to half a unit per SM, (8, 7) up to 2 units per SM, (8, 2)
-// below 12 per SM and (8, 1) above (76, 304 and 1824 units on a 152-SM
-// device), so that the GPU stays busy. The summation order depends on (S, B) and
-// differs from the one-warp-per-unit kernel, so all are chosen by launch
-// size alone -- every variant of a launch runs the same code -- and results
-// stay reproducible.
-constexpr int kSplitMaxWarps = 16;
+// K1 for small launches (few 64-pair units): the aperture of a unit's pairs is
+// cut into 8 B contiguous slices, whose partial sums are added eight at a time
+// in slice order and the B sums of eight in order. B is 9 up to half a unit
+// per SM, 7 up to 2 units per SM, 2 below 12 per SM and 1 above (76, 304 and
+// 1824 units on a 152-SM device). The summation order depends on B and differs
+// from the one-warp-per-unit kernel, so B is chosen by launch size alone --
+// every variant of a launch gives the same bits -- and results stay
+// reproducible. Two kernels run it, with the same bits:
+//  * k_semblance_split: a warp per slice, eight warps per block, a cluster of
+//    B blocks per unit. The blocks push their sums into the first one's shared
+//    memory and leave; no global scratch, fence, ticket or re-read. Latency
+//    bound (44% issue, 43% of the warps resident): a CRS launch of 118 units x
+//    1008 traces, w = 5, takes 30.9 us against 37.5 us through global scratch,
+//    258 units 63.0 us against 70.9 us, 24 units of 48 traces 9.7 against 12.5.
+//  * k_semblance_short: a warp per eight slices, walked one after the other,
+//    for apertures too short to feed 8 B warps (258 units x 48 traces: 10.4 us
+//    against 18.5 us with a warp per slice and 29.1 us through scratch).
+constexpr int kSplitWarps = 8;
 
-// warps per block of a one-block-per-unit split launch of `units` units on a
-// device of n_sm SMs: 8 once that keeps about 32 warps resident per SM, else 16
-inline int split_warps(long long units, int n_sm) {
-  return units * 8 >= (long long)n_sm * 32 ? 8 : kSplitMaxWarps;
+// Slice sl of nsl of a pair's aperture: entries floor(n sl / nsl) to
+// floor(n (sl + 1) / nsl), from n = h nsl + m in 32 bits (m sl < nsl^2).
+__device__ __forceinline__ void slice_of(const Lane& L, int nsl, int sl, int& r0, int& r1) {
+  const unsigned n = unsigned(L.e1 - L.e0), u = unsigned(nsl), h = n / u, m = n - h * u;
+  r0 = L.e0 + int(h * sl + m * sl / u);
+  r1 = L.e0 + int(h * (sl + 1) + m * (sl + 1) / u);
 }
 
-// Launches of at most n_sm * kSplitSmallPerSm units run kSplitMultiWarps warps per
-// block, kSplitSmallBlocks blocks per unit (56 slices per aperture), or
-// kSplitTinyBlocks (72 slices) up to n_sm / 2 units: 256-thread blocks, four
-// of which share an SM, so that one block's barrier overlaps the others'
-// loads. The best of the (S, B) pairs timed on the ENS 5 x 1 sweep, whose
-// launches hold 157 and 63 units (21.7 ms against 23.1 for (16, 4); (8, 5),
-// (8, 6), (8, 8), (16, 3), (16, 5) and for the smaller launches (8, 6),
-// (16, 4), (16, 8) were slower). Below n_sm * kSplitMultiPerSm units, (8, 2):
-// timed 17% faster than (8, 1) on the 938-unit launches of an ENS 30 x 30
-// sweep, while from about 2500 units (ENS 80 x 80) one block per unit is
-// best.
-constexpr int kSplitMultiWarps = 8;
+// What the end of a split launch needs of its unit's pairs: the aperture size
+// (-1 for an absent pair), kept in shared memory by one warp.
+__device__ __forceinline__ void keep_sizes(int* size, int lane, bool v0, const Lane& L0, bool v1,
+                                           const Lane& L1) {
+  size[lane] = v0 ? L0.e1 - L0.e0 : -1;
+  size[lane + 32] = v1 ? L1.e1 - L1.e0 : -1;
+}
 
-// dynamic shared memory of a split block: FP64 energies [S][64], FP32
-// energies [S][64], stack sums [S][64][K]
-inline size_t split_smem_bytes(int S, int W) {
-  return size_t(S) * 64 * (sizeof(double) + sizeof(float) + sizeof(float) * (2 * W + 1));
+// shared rows of 64 floats per set of sums: s_k and E; BF16 storage adds a row
+// of 64 doubles per set
+template <typename T>
+constexpr size_t split_set_bytes(int W) {
+  return 64 * (sizeof(float) * (2 * W + 2) + (Chunk<T>::kF64 ? sizeof(double) : 0));
+}
+// k_semblance_split: the block's eight slices, and (used by the cluster's
+// first block) the B blocks' sums
+inline size_t split_smem_bytes(int B, int W, bool bf16) {
+  const size_t set = bf16 ? split_set_bytes<__nv_bfloat16>(W) : split_set_bytes<float>(W);
+  return set * size_t(kSplitWarps + (B > 1 ? B : 0));
+}
+// k_semblance_short: the unit's B sums
+inline size_t short_smem_bytes(int B, int W, bool bf16) {
+  const size_t set = bf16 ? split_set_bytes<__nv_bfloat16>(W) : split_set_bytes<float>(W);
+  return set * size_t(B);
+}
+
+// S of pair q (row entry p) from its summed rows; N = -1 marks an absent pair.
+template <int W, typename T>
+__device__ __forceinline__ void finish_pair(const EvalArgs& a, long long q, int N,
+                                            const float* tot, double Ed) {
+  constexpr int K = 2 * W + 1;
+  if (N < 0) return;
+  float Q = 0.f;
+#pragma unroll
+  for (int k = 0; k < K; ++k) Q = fmaf(tot[k * 64], tot[k * 64], Q);
+  store_S(a, q, a.slots ? dom_of(q, a.P) : 0, normalise<T>(Q, N, tot[K * 64], Ed));
 }
 
 template <int OP, int W, typename T, bool MV>
-__global__ void __launch_bounds__(32 * kSplitMaxWarps, 2) k_semblance_split(const EvalArgs a) {
-  constexpr int K = 2 * W + 1;
+__global__ void __launch_bounds__(32 * kSplitWarps, 4) k_semblance_split(const EvalArgs a) {
+  constexpr int K = 2 * W + 1, R = K + 1;
+  constexpr int S = kSplitWarps, NT = 32 * S;
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cl = cg::this_cluster();
   extern __shared__ __align__(16) unsigned char split_smem[];
-  const int S = blockDim.x >> 5;
-  double* part_Ed = reinterpret_cast<double*>(split_smem);   // [S][64]
-  float* part_E = reinterpret_cast<float*>(part_Ed + S * 64);  // [S][64]
-  float* part_s = part_E + S * 64;                             // [S][64][K]
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int B = a.split_blocks;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const long long unit = blockIdx.x / B;
-  const int part = int(blockIdx.x - unit * B);
+  const int rank = int(blockIdx.x - unit * B);
+  double* part_Ed = reinterpret_cast<double*>(split_smem);  // [S][64], then [B][64]
+  double* recv_Ed = part_Ed + S * 64;
+  float* part = reinterpret_cast<float*>(part_Ed + (Chunk<T>::kF64 ? (S + (B > 1 ? B : 0)) * 64 : 0));
+  float* recv = part + S * R * 64;  // [B][R][64], in the cluster's first block
+  if (B > 1) cluster_arrive_relaxed();  // met by cluster_wait below: every block has started
   const long long q0 = unit * 64 + lane, q1 = q0 + 32;
   Lane L0, L1;
-  const bool v0 = lane_setup<OP>(a, q0, L0);
-  const bool v1 = lane_setup<OP>(a, q1, L1);
-  auto slice = [&](const Lane& L, int& r0, int& r1) {
-    const long long n = L.e1 - L.e0, nsl = (long long)S * B, sl = (long long)part * S + w;
-    r0 = L.e0 + int(n * sl / nsl);
-    r1 = L.e0 + int(n * (sl + 1) / nsl);
-  };
+  const bool v0 = lane_setup<OP, true>(a, q0, L0);
+  const bool v1 = lane_setup<OP, true>(a, q1, L1);
+  __shared__ int size[64];
+  if (w == 0) keep_sizes(size, lane, v0, L0, v1, L1);
+  const int nsl = S * B, sl = rank * S + w;
+  int r0, r1;
   if (v0 && v1 && same_aperture(L0, L1)) {
-    int r0, r1;
-    slice(L0, r0, r1);
+    slice_of(L0, nsl, sl, r0, r1);
     float2 s[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) s[k] = make_float2(0.f, 0.f);
@@ -473,88 +523,261 @@ __global__ void __launch_bounds__(32 * kSplitMaxWarps, 2) k_semblance_split(cons
     acc_packed<OP, W, T, MV>(a, L0, L1, r0, r1, s, E, Ed0, Ed1);
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-      part_s[(w * 64 + lane) * K + k] = s[k].x;
-      part_s[(w * 64 + lane + 32) * K + k] = s[k].y;
+      part[(w * R + k) * 64 + lane] = s[k].x;
+      part[(w * R + k) * 64 + lane + 32] = s[k].y;
     }
-    part_E[w * 64 + lane] = E.x;
-    part_E[w * 64 + lane + 32] = E.y;
-    part_Ed[w * 64 + lane] = Ed0;
-    part_Ed[w * 64 + lane + 32] = Ed1;
+    part[(w * R + K) * 64 + lane] = E.x;
+    part[(w * R + K) * 64 + lane + 32] = E.y;
+    if (Chunk<T>::kF64) {
+      part_Ed[w * 64 + lane] = Ed0;
+      part_Ed[w * 64 + lane + 32] = Ed1;
+    }
   } else {
     for (int h = 0; h < 2; ++h) {
-      const Lane& L = h ? L1 : L0;
-      if (!(h ? v1 : v0)) continue;
-      int r0, r1;
-      slice(L, r0, r1);
-      float s[K];
+      float s[K], E = 0.f;
+      double Ed = 0.0;
 #pragma unroll
       for (int k = 0; k < K; ++k) s[k] = 0.f;
-      float E = 0.f;
-      double Ed = 0.0;
-      acc_scalar<OP, W, T, MV>(a, L, r0, r1, s, E, Ed);
+      if (h ? v1 : v0) {
+        const Lane& L = h ? L1 : L0;
+        slice_of(L, nsl, sl, r0, r1);
+        acc_scalar<OP, W, T, MV>(a, L, r0, r1, s, E, Ed);
+      }
       const int p = lane + 32 * h;
 #pragma unroll
-      for (int k = 0; k < K; ++k) part_s[(w * 64 + p) * K + k] = s[k];
-      part_E[w * 64 + p] = E;
-      part_Ed[w * 64 + p] = Ed;
+      for (int k = 0; k < K; ++k) part[(w * R + k) * 64 + p] = s[k];
+      part[(w * R + K) * 64 + p] = E;
+      if (Chunk<T>::kF64) part_Ed[w * 64 + p] = Ed;
     }
   }
   __syncthreads();
-  // the block's sums of pair p = threadIdx.x (< 64), slices in order
-  const int p = threadIdx.x;
-  Lane L;
-  const bool valid = p < 64 && lane_setup<OP>(a, unit * 64 + p, L);
-  float sk[K];
-  float E = 0.f;
-  double Ed = 0.0;
+  // the block's sums, slices in order: to the cluster's first block
+  float* to = part;
+  double* to_d = part_Ed;
+  if (B > 1) {
+    cluster_wait();
+    to = cl.map_shared_rank(recv, 0) + rank * R * 64;
+    to_d = cl.map_shared_rank(recv_Ed, 0) + rank * 64;
+  }
+  for (int i = threadIdx.x; i < R * 64; i += NT) {
+    float t = 0.f;
 #pragma unroll
-  for (int k = 0; k < K; ++k) sk[k] = 0.f;
-  if (valid) {
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-      for (int v = 0; v < S; ++v) sk[k] = __fadd_rn(sk[k], part_s[(v * 64 + p) * K + k]);
-    for (int v = 0; v < S; ++v) {
-      E = __fadd_rn(E, part_E[v * 64 + p]);
-      Ed += part_Ed[v * 64 + p];
-    }
+    for (int v = 0; v < S; ++v) t = __fadd_rn(t, part[v * R * 64 + i]);
+    to[i] = t;
+  }
+  if (Chunk<T>::kF64 && threadIdx.x < 64) {
+    double t = 0.0;
+    for (int v = 0; v < S; ++v) t += part_Ed[v * 64 + threadIdx.x];
+    to_d[threadIdx.x] = t;
   }
   if (B > 1) {
-    // publish the block's sums; the unit's last block adds them in block order
-    const size_t set = size_t(unit) * B + part;
-    float* gp = a.split_part + (set * 64 + p) * kSplitPartStride;
-    if (valid) {
-#pragma unroll
-      for (int k = 0; k < K; ++k) gp[k] = sk[k];
-      gp[K] = E;
-      a.split_part_d[set * 64 + p] = Ed;
-    }
-    __threadfence();
-    __syncthreads();
-    __shared__ int last;
-    if (threadIdx.x == 0) last = atomicAdd(a.split_ticket + unit, 1u) == unsigned(B - 1);
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    if (threadIdx.x == 0) a.split_ticket[unit] = 0u;  // ready for the next launch
-    if (!valid) return;
-#pragma unroll
-    for (int k = 0; k < K; ++k) sk[k] = 0.f;
-    E = 0.f;
-    Ed = 0.0;
-    for (int b = 0; b < B; ++b) {
-      const size_t sb = size_t(unit) * B + b;
-      const float* q = a.split_part + (sb * 64 + p) * kSplitPartStride;
-#pragma unroll
-      for (int k = 0; k < K; ++k) sk[k] = __fadd_rn(sk[k], __ldcg(q + k));
-      E = __fadd_rn(E, __ldcg(q + K));
-      Ed += __ldcg(a.split_part_d + sb * 64 + p);
+    __syncwarp();
+    cluster_arrive();
+    if (rank) return;  // done with: nothing of this block's shared memory is read by others
+    cluster_wait();
+    for (int i = threadIdx.x; i < R * 64; i += NT) {
+      float t = 0.f;
+      for (int b = 0; b < B; ++b) t = __fadd_rn(t, recv[b * R * 64 + i]);
+      part[i] = t;
     }
   }
-  if (!valid) return;
-  float Q = 0.f;
+  __syncthreads();
+  if (threadIdx.x < 64) {
+    double Ed = 0.0;
+    if (Chunk<T>::kF64) {
+      if (B > 1)
+        for (int b = 0; b < B; ++b) Ed += recv_Ed[b * 64 + threadIdx.x];
+      else
+        Ed = part_Ed[threadIdx.x];
+    }
+    finish_pair<W, T>(a, unit * 64 + threadIdx.x, size[threadIdx.x], part + threadIdx.x, Ed);
+  }
+}
+
+// kSplitWarps consecutive slices of a pair's aperture, from slice sl0 of nsl:
+// entries e0 to e1, the first slice's end, and what the next ends take --
+// slice ends lie h or h + 1 entries apart, n = h nsl + m, as the remainder
+// `rem` of m times the slice number passes nsl. Set up once (the divisions
+// are as long as an entry's loads), walked without dividing.
+struct Slices {
+  int e0, e1, end, h, m, rem, nsl;
+  __device__ __forceinline__ void set(const Lane& L, int nsl_, int sl0) {
+    int r;
+    nsl = nsl_;
+    slice_of(L, nsl, sl0, e0, end);
+    slice_of(L, nsl, sl0 + kSplitWarps - 1, r, e1);
+    const int n = L.e1 - L.e0;
+    h = n / nsl;
+    m = n - h * nsl;
+    rem = m * (sl0 + 1) % nsl;
+  }
+  __device__ __forceinline__ void next() {
+    end += h;
+    rem += m;
+    if (rem >= nsl) {
+      rem -= nsl;
+      ++end;
+    }
+  }
+};
+
+// Sums of kSplitWarps consecutive slices of two pairs sharing an aperture, as
+// acc_packed gives each and added in slice order. Apertures of no more traces
+// than slices have at most one entry in a slice, whose amplitudes are the
+// slice's sums: they are added directly.
+template <int OP, int W, typename T, bool MV>
+__device__ __forceinline__ void acc_slices(const EvalArgs& a, const Lane& L0, const Lane& L1,
+                                           Slices at, float2* t, float2& tE, double& tEd0,
+                                           double& tEd1) {
+  constexpr int K = 2 * W + 1;
+  if (at.h == 0) {
+    const T* __restrict__ tr = static_cast<const T*>(a.traces);
+    for (int e = at.e0; e < at.e1; ++e) {
+      const float4 t4 = __ldg(a.ap_tab + e);
+      const Pos P0 = locate<OP, MV, true>(L0, t4), P1 = locate<OP, MV, true>(L1, t4);
+      const unsigned base = __float_as_uint(t4.w) - W;
+      const T* x0 = tr + (base + P0.j);
+      const T* x1 = tr + (base + P1.j);
+      float2 xv[K + 1];
 #pragma unroll
-  for (int k = 0; k < K; ++k) Q = fmaf(sk[k], sk[k], Q);
-  store_S(a, unit * 64 + p, L.d, normalise<T>(Q, L.e1 - L.e0, E, Ed));
+      for (int k = 0; k <= K; ++k) xv[k] = make_float2(ld_sample<T>(x0 + k), ld_sample<T>(x1 + k));
+      const float2 f = make_float2(P0.f, P1.f), g = make_float2(P0.g, P1.g);
+      float2 E = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const float2 ak = __ffma2_rn(f, xv[k + 1], __fmul2_rn(g, xv[k]));
+        t[k] = __fadd2_rn(t[k], ak);
+        E = __ffma2_rn(ak, ak, E);
+      }
+      if (Chunk<T>::kF64) {
+        tEd0 += double(E.x);
+        tEd1 += double(E.y);
+      } else {
+        tE = __fadd2_rn(tE, E);
+      }
+    }
+    return;
+  }
+  for (int v = 0, r0 = at.e0; v < kSplitWarps; ++v) {
+    float2 s[K], E = make_float2(0.f, 0.f);
+    double Ed0 = 0.0, Ed1 = 0.0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) s[k] = make_float2(0.f, 0.f);
+    acc_packed<OP, W, T, MV>(a, L0, L1, r0, at.end, s, E, Ed0, Ed1);
+#pragma unroll
+    for (int k = 0; k < K; ++k) t[k] = __fadd2_rn(t[k], s[k]);
+    tE = __fadd2_rn(tE, E);
+    tEd0 += Ed0;
+    tEd1 += Ed1;
+    r0 = at.end;
+    at.next();
+  }
+}
+
+// The same for one pair.
+template <int OP, int W, typename T, bool MV>
+__device__ __forceinline__ void acc_slices_scalar(const EvalArgs& a, const Lane& L, Slices at,
+                                                  float* t, float& tE, double& tEd) {
+  constexpr int K = 2 * W + 1;
+  for (int v = 0, r0 = at.e0; v < kSplitWarps; ++v) {
+    float s[K], E = 0.f;
+    double Ed = 0.0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) s[k] = 0.f;
+    acc_scalar<OP, W, T, MV>(a, L, r0, at.end, s, E, Ed);
+#pragma unroll
+    for (int k = 0; k < K; ++k) t[k] = __fadd_rn(t[k], s[k]);
+    tE = __fadd_rn(tE, E);
+    tEd += Ed;
+    r0 = at.end;
+    at.next();
+  }
+}
+
+// One of the unit's sums of eight slices, into row set `set` [K + 1][64] and
+// energies set_Ed [64]. A0, A1: the slices of the lane's pairs.
+template <int OP, int W, typename T, bool MV>
+__device__ __forceinline__ void unit_slices(const EvalArgs& a, bool v0, const Lane& L0,
+                                            const Slices& A0, bool v1, const Lane& L1,
+                                            const Slices& A1, int lane, float* set,
+                                            double* set_Ed) {
+  constexpr int K = 2 * W + 1;
+  if (v0 && v1 && same_aperture(L0, L1)) {
+    float2 t[K], E = make_float2(0.f, 0.f);
+    double Ed0 = 0.0, Ed1 = 0.0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) t[k] = make_float2(0.f, 0.f);
+    acc_slices<OP, W, T, MV>(a, L0, L1, A0, t, E, Ed0, Ed1);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      set[k * 64 + lane] = t[k].x;
+      set[k * 64 + lane + 32] = t[k].y;
+    }
+    set[K * 64 + lane] = E.x;
+    set[K * 64 + lane + 32] = E.y;
+    if (Chunk<T>::kF64) {
+      set_Ed[lane] = Ed0;
+      set_Ed[lane + 32] = Ed1;
+    }
+    return;
+  }
+  for (int h = 0; h < 2; ++h) {
+    float t[K], E = 0.f;
+    double Ed = 0.0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) t[k] = 0.f;
+    if (h ? v1 : v0)
+      acc_slices_scalar<OP, W, T, MV>(a, h ? L1 : L0, h ? A1 : A0, t, E, Ed);
+    const int p = lane + 32 * h;
+#pragma unroll
+    for (int k = 0; k < K; ++k) set[k * 64 + p] = t[k];
+    set[K * 64 + p] = E;
+    if (Chunk<T>::kF64) set_Ed[p] = Ed;
+  }
+}
+
+// The B sets of a unit added in order, into the first, by its 32 B threads.
+template <int W, int B>
+__device__ __forceinline__ void add_sets(float* set, int tid) {
+  constexpr int R = 2 * W + 2;
+#pragma unroll
+  for (int i0 = 0; i0 < R * 64; i0 += 32 * B) {
+    const int i = i0 + tid;
+    if (i >= R * 64) break;
+    float t = 0.f;
+#pragma unroll
+    for (int c = 0; c < B; ++c) t = __fadd_rn(t, set[c * R * 64 + i]);
+    set[i] = t;
+  }
+}
+
+template <int OP, int W, typename T, bool MV>
+__global__ void __launch_bounds__(32 * kSplitSmallBlocks, 2) k_semblance_short(const EvalArgs a) {
+  constexpr int B = kSplitSmallBlocks;
+  extern __shared__ __align__(16) unsigned char split_smem[];
+  __shared__ int size[64];
+  const int lane = threadIdx.x & 31, b = threadIdx.x >> 5;
+  const long long unit = blockIdx.x;
+  double* set_Ed = reinterpret_cast<double*>(split_smem);  // [B][64]
+  float* set = reinterpret_cast<float*>(set_Ed + (Chunk<T>::kF64 ? B * 64 : 0));
+  Lane L0, L1;
+  const bool v0 = lane_setup<OP, true>(a, unit * 64 + lane, L0);
+  const bool v1 = lane_setup<OP, true>(a, unit * 64 + lane + 32, L1);
+  if (b == 0) keep_sizes(size, lane, v0, L0, v1, L1);
+  Slices A0{}, A1{};
+  if (v0) A0.set(L0, kSplitWarps * B, kSplitWarps * b);
+  if (v1) A1.set(L1, kSplitWarps * B, kSplitWarps * b);
+  unit_slices<OP, W, T, MV>(a, v0, L0, A0, v1, L1, A1, lane, set + b * (2 * W + 2) * 64,
+                            set_Ed + b * 64);
+  __syncthreads();
+  add_sets<W, B>(set, threadIdx.x);
+  __syncthreads();
+  const int p = threadIdx.x;
+  if (p >= 64) return;
+  double Ed = 0.0;
+  if (Chunk<T>::kF64)
+    for (int c = 0; c < B; ++c) Ed += set_Ed[c * 64 + p];
+  finish_pair<W, T>(a, unit * 64 + p, size[p], set + p, Ed);
 }
 
 // K1, grid-mapped (queue == nullptr: one 64-pair unit per warp, the grid
@@ -809,7 +1032,7 @@ OFn pick_order(bool mv) {
 
 using SFn = void (*)(const EvalArgs, float*);
 enum KernelKind {
-  kKindPacked = 0, kKindScalar = 1, kKindSplit = 2, kKindGrad = 3
+  kKindPacked = 0, kKindScalar = 1, kKindSplit = 2, kKindGrad = 3, kKindShort = 6
 };
 
 template <int OP, int W, typename T, bool MV>
@@ -818,6 +1041,7 @@ KFn pick_kind(int kind) {
     case kKindPacked: return k_semblance<OP, W, T, MV>;
     case kKindScalar: return k_semblance_scalar<OP, W, T, MV>;
     case kKindSplit: return k_semblance_split<OP, W, T, MV>;
+    case kKindShort: return k_semblance_short<OP, W, T, MV>;
     case kKindGrad: return k_semblance_grad<OP, W, T, MV>;
   }
   return nullptr;

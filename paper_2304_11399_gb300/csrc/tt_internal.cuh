@@ -18,27 +18,14 @@ constexpr int op_dim(int op) { return op == TT_OP_CMP ? 1 : op == TT_OP_CRS ? 3 
 // Small-launch split thresholds, in 64-pair units per SM of the device
 // (the SM count is queried when a context is created): a forward launch of
 // fewer than n_sm * kSplitUnitsPerSm units (one warp per unit then leaves
-// SMs short of their 32 resident warps) splits each unit's aperture over
-// the warps of a block; up to n_sm * kSplitSmallPerSm units a unit spreads
-// over kSplitSmallBlocks blocks (kSplitTinyBlocks up to n_sm / 2 units),
-// below n_sm * kSplitMultiPerSm over two. The multi-block launches combine
-// partial sums in context scratch: one set per (unit, block), so the scratch
-// holds the largest units x blocks of any launch, at most
-// max(2 kSplitMultiPerSm, kSplitSmallPerSm kSplitSmallBlocks,
-// kSplitTinyBlocks / 2) n_sm sets.
+// SMs short of their 32 resident warps) splits each unit's aperture into 8 B
+// slices: B = kSplitTinyBlocks up to n_sm / 2 units, kSplitSmallBlocks up to
+// n_sm * kSplitSmallPerSm, 2 below n_sm * kSplitMultiPerSm, else 1.
 constexpr int kSplitUnitsPerSm = 32;
 constexpr int kSplitSmallPerSm = 2;
 constexpr int kSplitMultiPerSm = 12;
 constexpr int kSplitSmallBlocks = 7;
 constexpr int kSplitTinyBlocks = 9;
-static_assert(kSplitSmallPerSm * kSplitSmallBlocks <= 2 * kSplitMultiPerSm &&
-                  kSplitTinyBlocks <= 4 * kSplitMultiPerSm,
-              "every split shape fits the 2 kSplitMultiPerSm n_sm part sets");
-// scratch sets (one per block of a multi-block split launch) and tickets
-// (one per unit) for a device of n_sm SMs
-inline long long split_part_sets(int n_sm) { return 2ll * kSplitMultiPerSm * n_sm; }
-inline long long split_tickets(int n_sm) { return (long long)kSplitMultiPerSm * n_sm; }
-constexpr int kSplitPartStride = 2 * 8 + 2;  // floats per pair: K + 1 for the widest window
 
 // Padded trace layout: sample n of trace r lives at r * pitch + kPadFront + n.
 // kPadFront >= max half window; kPadBack >= 2 * max half window + 2 so that a
@@ -46,6 +33,7 @@ constexpr int kSplitPartStride = 2 * 8 + 2;  // floats per pair: K + 1 for the w
 constexpr int kPadFront = 8;
 constexpr int kPadBack = 24;
 constexpr int kBlock = 256;
+constexpr int kProbeFloats = 8192 + 1;
 constexpr int kOrderMaxP = 256;  // largest population the member order handles
 // automatic member order: on when the mean aperture holds at least this many traces
 constexpr double kOrderMinMeanAperture = 768.0;
@@ -71,11 +59,8 @@ struct EvalArgs {
   int kernel;               // TT_KERNEL_PACKED / _PERSISTENT / _SCALAR (forward launches)
   int block;                // threads per block: 128 or 256
   int split;                // 1: small forward launches split the aperture over warps
-  int split_blocks;         // blocks per unit of a split launch (set by the launcher)
+  int split_blocks;         // B of a split launch (set by the launcher)
   int n_sm;                 // SMs of the device (split thresholds, persistent grid)
-  float* split_part;        // [split_part_sets][64][K + 1] block partial sums (s_k, E)
-  double* split_part_d;     // [split_part_sets][64] block partial FP64 energies
-  unsigned* split_ticket;   // [split_tickets] arrivals per unit, zero between launches
   unsigned long long* queue;  // persistent mode: work-unit counter, zero at launch
   int n_groups;             // aperture groups of the context
   float mean_ap;            // mean aperture size over the context's domains
@@ -227,14 +212,9 @@ struct tt_ctx {
         *pol_bS = nullptr;
   int* d_err = nullptr;     // device-side validation flag
   unsigned long long* queue = nullptr;  // persistent-kernel work counter
-  float* split_part = nullptr;          // multi-block split scratch (tt::split_part_sets sets)
-  double* split_part_d = nullptr;
-  unsigned* split_ticket = nullptr;
-  // a second split scratch and a side stream: the ENS sweep evaluates each
-  // step's interpolated samples concurrently with the next step
-  float* split_part2 = nullptr;
-  double* split_part_d2 = nullptr;
-  unsigned* split_ticket2 = nullptr;
+  float* probe = nullptr;   // window and sink of the L1 probe (kProbeFloats)
+  // a side stream: the ENS sweep evaluates each step's interpolated samples
+  // concurrently with the next step
   cudaStream_t side_stream = nullptr;
   cudaEvent_t side_ev[4] = {nullptr, nullptr, nullptr, nullptr};
   // launch configuration (tt_ctx_set_option / tt_ctx_autotune)

@@ -56,3 +56,29 @@ def test_stack_lane_and_warp_per_domain_bit_identical(n_dom, sizes, ns, storage)
         outs.append(tt.tt_stack(ctx, th))
         ctx.close()
     assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("op,w,storage,ns,sizes", [
+    (1, 5, "f32", 300, (100,)), (1, 0, "f32", 2200, (57, 143)), (2, 8, "bf16", 300, (99, 101)),
+    (1, 3, "bf16", 300, (300, 1, 0, 99))])
+def test_slices_walked_by_one_warp_or_eight(op, w, storage, ns, sizes):
+    """A launch of 160 units and one of 176 cut apertures into the same 56
+    slices, the first with a warp per slice, the second (mean aperture under
+    0.6 per unit) with a warp per eight: the members they share have the same
+    S bit for bit. 300 entries are more than 56 chunks of 32 would hold
+    per slice of one entry; 57 to 143 leave slices of one to three, 1 and 0
+    leave most or all empty."""
+    n_dom = 1024
+    x, mid, off = _line(60, ns)
+    prob = _problem(n_dom, sizes, 60, ns, op, w)
+    th = to_dev(random_theta(n_dom, 11, *BOUNDS[op], 7))
+    ctx = tt.tt_ctx_create(x, mid, off, prob, None, storage=storage, device=dev())
+    if tt.tt_ctx_get_option(ctx, "sm_count") != 152:
+        pytest.skip("launch sizes chosen for 152 multiprocessors")
+    a = tt.tt_semblance_eval(ctx, th[:, :10].contiguous())
+    b = tt.tt_semblance_eval(ctx, th)
+    ctx.close()
+    assert torch.equal(a, b[:, :10])
+    if storage == "f32":
+        ref = oracle.semblance.semblance_many(x, mid, off, prob, th[:, :2].cpu().numpy())
+        assert np.max(np.abs(a[:, :2].cpu().numpy() - ref)) <= 1e-5
