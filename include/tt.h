@@ -338,7 +338,9 @@ tt_status tt_ctx_probe_l1(tt_ctx* ctx, int32_t iters, double* bytes, void* strea
  *                 slice order; every variant then sums alike, so S
  *                 still does not depend on TT_OPT_KERNEL / TT_OPT_BLOCK, but
  *                 its rounding differs from the unsplit kernels' (all stay
- *                 within 1e-5 of the exact semblance). 0: never split.
+ *                 within 1e-5 of the exact semblance). Gradient evaluations are
+ *                 split too (tt_semblance_grad; not inside the polish, whose
+ *                 iterates are compared by their S). 0: never split.
  *  TT_OPT_MEMBER_ORDER  1: before each generation's evaluation inside
  *                 tt_search / tt_search_slab (NP <= 256), the members of
  *                 every domain are put in the order of their window position

@@ -85,6 +85,43 @@ cudaError_t launch_split(EvalArgs& a, long long units, bool mv, cudaStream_t s) 
   return cudaLaunchKernelEx(&cfg, fn, a);
 }
 
+// Split gradient launches: with apertures of 256 traces or more at every size
+// (1008 traces: 24 / 938 / 9375 units 28 / 474 / 3763 us against 740 / 839 /
+// 4101 us with one pair per thread), with shorter ones down to 16 traces while
+// the launch has fewer than 16 units per SM (144 traces: 469 units 75 us
+// against 98 us, 4688 units 322 us against 307 us; 48 traces: 16 units 18 us
+// against 50 us, 9375 units 284 us against 217 us).
+bool grad_split(const EvalArgs& a, long long units) {
+  return a.split && (a.mean_ap >= 256.f || (a.mean_ap >= 16.f && units < 16ll * a.n_sm));
+}
+
+// The cluster grows to 8 blocks while the launch has fewer than 7 blocks per SM
+// (three run on an SM at a time, so that the last wave weighs little) and the
+// slices hold 4 traces on average (1008 traces, clusters of 1 / 2 / 4 / 8: 24
+// units 115 / 66 / 38 / 28 us, 282 units 308 / 235 / 207 / 217 us, 938 units
+// 647 / 562 / 577 / 680 us, at two blocks per SM).
+cudaError_t launch_grad_split(const EvalArgs& a, long long units, bool mv, cudaStream_t s) {
+  const KFn fn = pick(sk::kKindGradSplit, a, mv);
+  if (!fn) return cudaErrorInvalidValue;
+  int B = 1;
+  while (B < sk::kGradMaxCluster && units * B < 7ll * a.n_sm &&
+         a.mean_ap >= float(4 * sk::kGradWarps * B))
+    B *= 2;
+  if (units * B > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = unsigned(B);
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(units * B));
+  cfg.blockDim = dim3(32 * sk::kGradWarps);
+  cfg.dynamicSmemBytes = sk::grad_smem_bytes(a.W, op_dim(a.op));
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, a);
+}
+
 cudaError_t launch(const EvalArgs& a, cudaStream_t s, bool grad) {
   const long long n = (long long)a.n_dom * a.P;
   if (n == 0) return cudaSuccess;
@@ -95,8 +132,17 @@ cudaError_t launch(const EvalArgs& a, cudaStream_t s, bool grad) {
   long long blocks;
   EvalArgs b = a;
   if (grad) {
-    fn = pick(sk::kKindGrad, a, mv);
-    blocks = (n + block - 1) / block;
+    const long long units = (n + 63) / 64;
+      if (grad_split(a, units)) return launch_grad_split(a, units, mv, s);
+    // few pairs: several entries in flight, in small blocks that spread over the SMs
+    const bool few = n < 768ll * a.n_sm;
+    fn = pick(few ? sk::kKindGradAhead : sk::kKindGrad, a, mv);
+    if (!fn) return cudaErrorInvalidValue;
+    const int threads = few ? 32 : 128;
+    blocks = (n + threads - 1) / threads;
+    if (blocks > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+    fn<<<unsigned(blocks), threads, 0, s>>>(a);
+    return cudaGetLastError();
   } else if (a.split && (n + 63) / 64 < (long long)a.n_sm * kSplitUnitsPerSm) {
     // too few units to fill the GPU: each unit's aperture split over warps
     return launch_split(b, (n + 63) / 64, mv, s);

@@ -69,6 +69,12 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
   return y;
 }
 
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 template <typename T>
 __device__ __forceinline__ float ld_sample(const T* p);
 template <>
@@ -814,49 +820,190 @@ __global__ void __launch_bounds__(kBlock) k_semblance_scalar(const EvalArgs a) {
 // forms dS/du_i = sum_k (alpha s_k - beta a_ik)(x[j+k+1] - x[j+k]) and
 // chains it through du/dtheta (u = p0 + du in samples, q = p0 + A' dm):
 //   du/dA = q dm / (u dt),  du/dB = dm^2 / (2 u dt^2),  du/dC = h^2 / (2 u dt^2).
-// Positions clamped to the all-zero window and u = 0 contribute nothing.
+// u = 0 contributes nothing, and positions clamped to the all-zero window give
+// zero by themselves.
+
+// d S / d u of one trace over u: the factor every parameter's chain shares.
+__device__ __forceinline__ float over_u(float dSdu, float u) {
+  return u > 0.f ? __fmul_rn(dSdu, rcp_approx(u)) : 0.f;
+}
+
+// Pass 2 of one pair over aperture entries [r0, r1): G += the entries' terms
+// (without the 1/dt factors). nbeta = -beta.
 template <int OP, int W, typename T, bool MV>
-__global__ void __launch_bounds__(kBlock) k_semblance_grad(const EvalArgs a) {
+__device__ __forceinline__ void adj_scalar(const EvalArgs& a, const Lane& L, int r0, int r1,
+                                           const float* s, float alpha, float nbeta, float* G) {
   constexpr int K = 2 * W + 1;
-  constexpr int D = op_dim(OP);
-  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  Lane L;
-  if (!lane_setup<OP>(a, q, L)) return;
   const T* __restrict__ tr = static_cast<const T*>(a.traces);
-  float s[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) s[k] = 0.f;
-  float E = 0.f;
-  for (int e = L.e0; e < L.e1; ++e) {
+  for (int e = r0; e < r1; ++e) {
     const float4 t4 = __ldg(a.ap_tab + e);
     const Pos P = locate<OP, MV>(L, t4);
     const T* x = tr + (__float_as_uint(t4.w) + P.j - W);
     float xv[K + 1];
 #pragma unroll
     for (int k = 0; k <= K; ++k) xv[k] = ld_sample<T>(x + k);
+    float sg = 0.f, ag = 0.f;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const float gk = __fsub_rn(xv[k + 1], xv[k]);
+      const float ak = fmaf(P.f, xv[k + 1], __fmul_rn(P.g, xv[k]));
+      sg = fmaf(s[k], gk, sg);
+      ag = fmaf(ak, gk, ag);
+    }
+    const float c = over_u(fmaf(alpha, sg, __fmul_rn(nbeta, ag)), P.u);
+    const float hc = __fmul_rn(0.5f, c), cq = __fmul_rn(c, P.q);
+    if (OP == TT_OP_FOCRS) {  // dU = 2q dm, 2q dh, dm^2, dm dh, dh^2
+      const float hm = __fmul_rn(hc, t4.x), hh = __fmul_rn(hc, t4.y);
+      G[0] = fmaf(cq, t4.x, G[0]);
+      G[1] = fmaf(cq, t4.y, G[1]);
+      G[2] = fmaf(hm, t4.x, G[2]);
+      G[3] = fmaf(hm, t4.y, G[3]);
+      G[4] = fmaf(hh, t4.y, G[4]);
+    } else if (OP == TT_OP_CRS) {
+      G[0] = fmaf(cq, t4.x, G[0]);
+      G[1] = fmaf(hc, t4.y, G[1]);
+      G[2] = fmaf(hc, t4.z, G[2]);
+    } else {
+      G[0] = fmaf(hc, t4.z, G[0]);
+    }
+  }
+}
+
+// The same for two pairs sharing an aperture, with packed FP32x2 arithmetic.
+template <int OP, int W, typename T, bool MV>
+__device__ __forceinline__ void adj_packed(const EvalArgs& a, const Lane& L0, const Lane& L1,
+                                           int r0, int r1, const float2* s, float2 alpha,
+                                           float2 nbeta, float2* G) {
+  constexpr int K = 2 * W + 1;
+  const T* __restrict__ tr = static_cast<const T*>(a.traces);
+  const float2 m1 = make_float2(-1.f, -1.f), half = make_float2(0.5f, 0.5f);
+  for (int e = r0; e < r1; ++e) {
+    const float4 t4 = __ldg(a.ap_tab + e);
+    const Pos P0 = locate<OP, MV>(L0, t4), P1 = locate<OP, MV>(L1, t4);
+    const unsigned base = __float_as_uint(t4.w) - W;
+    const T* x0 = tr + (base + P0.j);
+    const T* x1 = tr + (base + P1.j);
+    float2 xv[K + 1];
+#pragma unroll
+    for (int k = 0; k <= K; ++k) xv[k] = make_float2(ld_sample<T>(x0 + k), ld_sample<T>(x1 + k));
+    const float2 f = make_float2(P0.f, P1.f), g = make_float2(P0.g, P1.g);
+    float2 sg = make_float2(0.f, 0.f), ag = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const float2 gk = __ffma2_rn(xv[k], m1, xv[k + 1]);
+      const float2 ak = __ffma2_rn(f, xv[k + 1], __fmul2_rn(g, xv[k]));
+      sg = __ffma2_rn(s[k], gk, sg);
+      ag = __ffma2_rn(ak, gk, ag);
+    }
+    const float2 d = __ffma2_rn(alpha, sg, __fmul2_rn(nbeta, ag));
+    const float2 c = make_float2(over_u(d.x, P0.u), over_u(d.y, P1.u));
+    const float2 hc = __fmul2_rn(half, c), cq = __fmul2_rn(c, make_float2(P0.q, P1.q));
+    const float2 tx = make_float2(t4.x, t4.x), ty = make_float2(t4.y, t4.y),
+                 tz = make_float2(t4.z, t4.z);
+    if (OP == TT_OP_FOCRS) {
+      const float2 hm = __fmul2_rn(hc, tx), hh = __fmul2_rn(hc, ty);
+      G[0] = __ffma2_rn(cq, tx, G[0]);
+      G[1] = __ffma2_rn(cq, ty, G[1]);
+      G[2] = __ffma2_rn(hm, tx, G[2]);
+      G[3] = __ffma2_rn(hm, ty, G[3]);
+      G[4] = __ffma2_rn(hh, ty, G[4]);
+    } else if (OP == TT_OP_CRS) {
+      G[0] = __ffma2_rn(cq, tx, G[0]);
+      G[1] = __ffma2_rn(hc, ty, G[1]);
+      G[2] = __ffma2_rn(hc, tz, G[2]);
+    } else {
+      G[0] = __ffma2_rn(hc, tz, G[0]);
+    }
+  }
+}
+
+// S, alpha and -beta from a pair's sums (all zero when the energy is 0).
+template <typename T>
+__device__ __forceinline__ float grad_factors(float Q, int N, float E, double Ed, float& alpha,
+                                              float& nbeta) {
+  const float S = normalise<T>(Q, N, E, Ed);
+  const float En = Chunk<T>::kF64 ? float(Ed) : E;
+  const bool ok = En > 0.f;
+  alpha = ok ? 2.f / (float(N) * En) : 0.f;
+  nbeta = ok ? -2.f * S / En : 0.f;
+  return S;
+}
+
+// dS of pair q: the 1/dt factors; zero when the energy is 0 (alpha = 0).
+template <int OP>
+__device__ __forceinline__ void store_grad(const EvalArgs& a, long long q, float inv_dt,
+                                           float alpha, const float* G) {
+  constexpr int D = op_dim(OP);
+  constexpr int n1 = OP == TT_OP_FOCRS ? 2 : OP == TT_OP_CRS ? 1 : 0;  // slopes: 1/dt
+  const float i2 = inv_dt * inv_dt;
+  float* out = a.dS + q * D;
+#pragma unroll
+  for (int d = 0; d < D; ++d) out[d] = alpha > 0.f ? G[d] * (d < n1 ? inv_dt : i2) : 0.f;
+}
+
+// K2 with one pair per thread, both passes in entry order: the form of the
+// polish (which compares the S of successive iterates, so its sums may not
+// depend on the launch), of splitting off and of short apertures. U entries
+// are in flight at a time: their table rows, positions and windows are loaded
+// before the first is added. A small launch of one pair per domain has few
+// warps to hide an L2 load behind and takes U = 6 (1008 traces, w = 5, 1,500 /
+// 60,000 domains: one entry at a time 808 / 956 us, two 563 / 761, four 412 /
+// 623, six 364 / 581); a large one has the warps and takes U = 1 (300,000
+// domains 2126 us, four at a time 2305 us). U does not change a bit.
+template <int OP, int W, typename T, bool MV, int U, typename F>
+__device__ __forceinline__ void each_window(const EvalArgs& a, const Lane& L, F&& add) {
+  constexpr int K = 2 * W + 1;
+  const T* __restrict__ tr = static_cast<const T*>(a.traces);
+  for (int e = L.e0; e < L.e1; e += U) {
+    float4 t4[U];
+    Pos P[U];
+    float xv[U][K + 1];
+#pragma unroll
+    for (int v = 0; v < U; ++v) t4[v] = __ldg(a.ap_tab + min(e + v, L.e1 - 1));
+#pragma unroll
+    for (int v = 0; v < U; ++v) {
+      P[v] = locate<OP, MV, true>(L, t4[v]);
+      const T* x = tr + (__float_as_uint(t4[v].w) + P[v].j - W);
+#pragma unroll
+      for (int k = 0; k <= K; ++k) xv[v][k] = ld_sample<T>(x + k);
+    }
+#pragma unroll
+    for (int v = 0; v < U; ++v)
+      if (e + v < L.e1) add(t4[v], P[v], xv[v]);
+  }
+}
+
+template <int OP, int W, typename T, bool MV, int U>
+__global__ void __launch_bounds__(128) k_semblance_grad(const EvalArgs a) {
+  constexpr int K = 2 * W + 1;
+  constexpr int D = op_dim(OP);
+  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  Lane L;
+  if (!lane_setup<OP>(a, q, L)) return;
+  float s[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) s[k] = 0.f;
+  float E = 0.f;
+  each_window<OP, W, T, MV, U>(a, L, [&](float4, const Pos& P, const float* xv) {
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       const float ak = fmaf(P.f, xv[k + 1], __fmul_rn(P.g, xv[k]));
       s[k] += ak;
       E = fmaf(ak, ak, E);
     }
-  }
+  });
   float Q = 0.f;
 #pragma unroll
   for (int k = 0; k < K; ++k) Q = fmaf(s[k], s[k], Q);
   const float N = float(L.e1 - L.e0);
   const float S = (E > 0.f) ? Q / (N * E) : 0.f;
-  float G0 = 0.f, G1 = 0.f, G2 = 0.f, G3 = 0.f, G4 = 0.f;
+  float G[D];
+#pragma unroll
+  for (int d = 0; d < D; ++d) G[d] = 0.f;
   if (E > 0.f) {
     const float alpha = 2.f / (N * E);
     const float beta = 2.f * S / E;
-    for (int e = L.e0; e < L.e1; ++e) {
-      const float4 t4 = __ldg(a.ap_tab + e);
-      const Pos P = locate<OP, MV>(L, t4);
-      const T* x = tr + (__float_as_uint(t4.w) + P.j - W);
-      float xv[K + 1];
-#pragma unroll
-      for (int k = 0; k <= K; ++k) xv[k] = ld_sample<T>(x + k);
+    each_window<OP, W, T, MV, U>(a, L, [&](float4 t4, const Pos& P, const float* xv) {
       float sg = 0.f, ag = 0.f;
 #pragma unroll
       for (int k = 0; k < K; ++k) {
@@ -869,36 +1016,207 @@ __global__ void __launch_bounds__(kBlock) k_semblance_grad(const EvalArgs a) {
       const float inv_u = (P.u > 0.f && P.u < L.umax) ? 1.f / P.u : 0.f;
       const float c = dSdu * inv_u;
       if (OP == TT_OP_FOCRS) {  // dU = 2q dm, 2q dh, dm^2, dm dh, dh^2
-        G0 = fmaf(c * P.q, t4.x, G0);
-        G1 = fmaf(c * P.q, t4.y, G1);
-        G2 = fmaf(0.5f * c, t4.x * t4.x, G2);
-        G3 = fmaf(0.5f * c, t4.x * t4.y, G3);
-        G4 = fmaf(0.5f * c, t4.y * t4.y, G4);
-        continue;
+        G[0] = fmaf(c * P.q, t4.x, G[0]);
+        G[1] = fmaf(c * P.q, t4.y, G[1]);
+        G[2] = fmaf(0.5f * c, t4.x * t4.x, G[2]);
+        G[3] = fmaf(0.5f * c, t4.x * t4.y, G[3]);
+        G[4] = fmaf(0.5f * c, t4.y * t4.y, G[4]);
+      } else if (OP == TT_OP_CRS) {
+        G[0] = fmaf(c * P.q, t4.x, G[0]);
+        G[1] = fmaf(0.5f * c, t4.y, G[1]);
+        G[2] = fmaf(0.5f * c, t4.z, G[2]);
+      } else {
+        G[0] = fmaf(0.5f * c, t4.z, G[0]);
       }
-      if (OP == TT_OP_CRS) {
-        G0 = fmaf(c * P.q, t4.x, G0);
-        G1 = fmaf(0.5f * c, t4.y, G1);
-      }
-      G2 = fmaf(0.5f * c, t4.z, G2);
-    }
+    });
   }
   a.S[q] = S;
-  float* out = a.dS + q * D;
+  constexpr int n1 = OP == TT_OP_FOCRS ? 2 : OP == TT_OP_CRS ? 1 : 0;  // slopes: 1/dt
   const float i2 = L.inv_dt * L.inv_dt;
-  if (OP == TT_OP_FOCRS) {
-    out[0] = G0 * L.inv_dt;
-    out[1] = G1 * L.inv_dt;
-    out[2] = G2 * i2;
-    out[3] = G3 * i2;
-    out[4] = G4 * i2;
-  } else if (OP == TT_OP_CRS) {
-    out[0] = G0 * L.inv_dt;
-    out[1] = G1 * i2;
-    out[2] = G2 * i2;
+#pragma unroll
+  for (int d = 0; d < D; ++d) a.dS[q * D + d] = G[d] * (d < n1 ? L.inv_dt : i2);
+}
+
+// K2 split: a cluster of B blocks of kGradWarps warps shares one 64-pair unit,
+// warp w of block b walking slice b kGradWarps + w of every pair's aperture in
+// both passes. Each pass's partial sums meet in shared memory (slices in
+// order) and across the cluster's blocks through distributed shared memory
+// (blocks in order); the cluster barriers take the place of a second launch.
+// The gradient usually has one pair per domain, so that a thread per pair
+// leaves a few warps per SM, each waiting on 1008 x 2 dependent window loads:
+// 60,000 CRS domains, 1008 traces, w = 5: 962 us, now 474 us; 1500 domains 835
+// us, now 28 us. Three blocks per SM (80 registers) hide more load latency
+// than two (102 registers: 562 us); it stays bound by its window loads (two
+// passes at K1's rate).
+constexpr int kGradWarps = 8;
+constexpr int kGradMaxCluster = 8;
+
+// shared memory of a block: FP64 energies [kGradWarps + 1][64]; rows of 64
+// floats that hold the slice sums of s and E [kGradWarps][K + 1], later the
+// unit's s and E, alpha, -beta and the slices' G [kGradWarps][D]; and the
+// block's sums [K + 1] (later its G [D])
+constexpr int grad_rows(int W, int D) {
+  const int R = 2 * W + 2, first = kGradWarps * R, second = R + 2 + kGradWarps * D;
+  return first > second ? first : second;
+}
+constexpr size_t grad_smem_bytes(int W, int D) {
+  const int R = 2 * W + 2;
+  return 64 * (sizeof(float) * size_t(grad_rows(W, D) + (R > D ? R : D)) +
+               sizeof(double) * size_t(kGradWarps + 1));
+}
+static_assert(grad_smem_bytes(TT_MAX_HALF_WINDOW, 5) <= 48 * 1024, "fits without an opt-in");
+
+template <int OP, int W, typename T, bool MV>
+__global__ void __launch_bounds__(32 * kGradWarps, 3) k_semblance_grad_split(const EvalArgs a) {
+  constexpr int K = 2 * W + 1, R = K + 1;  // R rows of 64: s_k and E
+  constexpr int D = op_dim(OP);
+  constexpr int S = kGradWarps, NT = 32 * S;
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cl = cg::this_cluster();
+  extern __shared__ __align__(16) unsigned char grad_smem[];
+  double* part_Ed = reinterpret_cast<double*>(grad_smem);      // [S][64]
+  double* blk_Ed = part_Ed + S * 64;                           // [64]
+  float* part = reinterpret_cast<float*>(blk_Ed + 64);         // [S][R][64]
+  float* blk = part + grad_rows(W, D) * 64;                    // [R][64]
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int B = int(cl.num_blocks()), rank = int(cl.block_rank());
+  const long long unit = blockIdx.x / B;
+  const long long q0 = unit * 64 + lane, q1 = q0 + 32;
+  Lane L0, L1;
+  const bool v0 = lane_setup<OP, true>(a, q0, L0), v1 = lane_setup<OP, true>(a, q1, L1);
+  const bool both = v0 && v1 && same_aperture(L0, L1);
+  __shared__ int size[64];
+  if (w == 0) keep_sizes(size, lane, v0, L0, v1, L1);
+  // pass 1
+  int r0 = 0, r1 = 0;
+  if (both) {
+    slice_of(L0, S * B, rank * S + w, r0, r1);
+    float2 s[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) s[k] = make_float2(0.f, 0.f);
+    float2 E = make_float2(0.f, 0.f);
+    double Ed0 = 0.0, Ed1 = 0.0;
+    acc_packed<OP, W, T, MV>(a, L0, L1, r0, r1, s, E, Ed0, Ed1);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      part[(w * R + k) * 64 + lane] = s[k].x;
+      part[(w * R + k) * 64 + lane + 32] = s[k].y;
+    }
+    part[(w * R + K) * 64 + lane] = E.x;
+    part[(w * R + K) * 64 + lane + 32] = E.y;
+    if (Chunk<T>::kF64) {
+      part_Ed[w * 64 + lane] = Ed0;
+      part_Ed[w * 64 + lane + 32] = Ed1;
+    }
   } else {
-    out[0] = G2 * i2;
+    for (int h = 0; h < 2; ++h) {
+      float s[K], E = 0.f;
+      double Ed = 0.0;
+#pragma unroll
+      for (int k = 0; k < K; ++k) s[k] = 0.f;
+      if (h ? v1 : v0) {
+        const Lane& L = h ? L1 : L0;
+        slice_of(L, S * B, rank * S + w, r0, r1);
+        acc_scalar<OP, W, T, MV>(a, L, r0, r1, s, E, Ed);
+      }
+      const int p = lane + 32 * h;
+#pragma unroll
+      for (int k = 0; k < K; ++k) part[(w * R + k) * 64 + p] = s[k];
+      part[(w * R + K) * 64 + p] = E;
+      if (Chunk<T>::kF64) part_Ed[w * 64 + p] = Ed;
+    }
   }
+  __syncthreads();
+  for (int i = threadIdx.x; i < R * 64; i += NT) {
+    float t = 0.f;
+#pragma unroll
+    for (int v = 0; v < S; ++v) t = __fadd_rn(t, part[v * R * 64 + i]);
+    blk[i] = t;
+  }
+  if (Chunk<T>::kF64 && threadIdx.x < 64) {
+    double t = 0.0;
+    for (int v = 0; v < S; ++v) t += part_Ed[v * 64 + threadIdx.x];
+    blk_Ed[threadIdx.x] = t;
+  }
+  if (B > 1) cl.sync(); else __syncthreads();
+  // the unit's sums, in every block, over the slice sums that are done with
+  float* tot = part;                     // [R][64]
+  float* fac = part + R * 64;            // alpha [64], -beta [64]
+  float* gsl = fac + 2 * 64;             // [S][D][64]
+  for (int i = threadIdx.x; i < R * 64; i += NT) {
+    float t = 0.f;
+    for (int b = 0; b < B; ++b) t = __fadd_rn(t, B > 1 ? cl.map_shared_rank(blk, b)[i] : blk[i]);
+    tot[i] = t;
+  }
+  __syncthreads();
+  if (threadIdx.x < 64 && size[threadIdx.x] >= 0) {
+    const int p = threadIdx.x;
+    float Q = 0.f, al, nb;
+#pragma unroll
+    for (int k = 0; k < K; ++k) Q = fmaf(tot[k * 64 + p], tot[k * 64 + p], Q);
+    double Ed = 0.0;
+    if (Chunk<T>::kF64)
+      for (int b = 0; b < B; ++b) Ed += B > 1 ? cl.map_shared_rank(blk_Ed, b)[p] : blk_Ed[p];
+    const float Sv = grad_factors<T>(Q, size[p], tot[K * 64 + p], Ed, al, nb);
+    fac[p] = al;
+    fac[64 + p] = nb;
+    if (rank == 0) a.S[unit * 64 + p] = Sv;
+  }
+  if (B > 1) cl.sync(); else __syncthreads();  // every block has read blk: it is free
+  // pass 2
+  if (both) {
+    float2 s[K], G[D];
+#pragma unroll
+    for (int k = 0; k < K; ++k) s[k] = make_float2(tot[k * 64 + lane], tot[k * 64 + lane + 32]);
+#pragma unroll
+    for (int d = 0; d < D; ++d) G[d] = make_float2(0.f, 0.f);
+    adj_packed<OP, W, T, MV>(a, L0, L1, r0, r1, s, make_float2(fac[lane], fac[lane + 32]),
+                             make_float2(fac[64 + lane], fac[96 + lane]), G);
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      gsl[(w * D + d) * 64 + lane] = G[d].x;
+      gsl[(w * D + d) * 64 + lane + 32] = G[d].y;
+    }
+  } else {
+    for (int h = 0; h < 2; ++h) {
+      const int p = lane + 32 * h;
+      float s[K], G[D];
+#pragma unroll
+      for (int d = 0; d < D; ++d) G[d] = 0.f;
+      if (h ? v1 : v0) {
+        const Lane& L = h ? L1 : L0;
+        slice_of(L, S * B, rank * S + w, r0, r1);
+#pragma unroll
+        for (int k = 0; k < K; ++k) s[k] = tot[k * 64 + p];
+        adj_scalar<OP, W, T, MV>(a, L, r0, r1, s, fac[p], fac[64 + p], G);
+      }
+#pragma unroll
+      for (int d = 0; d < D; ++d) gsl[(w * D + d) * 64 + p] = G[d];
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < D * 64; i += NT) {
+    float t = 0.f;
+#pragma unroll
+    for (int v = 0; v < S; ++v) t = __fadd_rn(t, gsl[v * D * 64 + i]);
+    blk[i] = t;
+  }
+  if (B > 1) cl.sync(); else __syncthreads();
+  if (rank == 0 && threadIdx.x < 64) {
+    const int p = threadIdx.x;
+    Lane L;
+    if (lane_setup<OP>(a, unit * 64 + p, L)) {
+      float G[D];
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        G[d] = 0.f;
+        for (int b = 0; b < B; ++b)
+          G[d] = __fadd_rn(G[d], B > 1 ? cl.map_shared_rank(blk, b)[d * 64 + p] : blk[d * 64 + p]);
+      }
+      store_grad<OP>(a, unit * 64 + p, L.inv_dt, fac[p], G);
+    }
+  }
+  if (B > 1) cl.sync();  // no block leaves while another may read its sums
 }
 
 using KFn = void (*)(const EvalArgs);
@@ -1032,7 +1350,8 @@ OFn pick_order(bool mv) {
 
 using SFn = void (*)(const EvalArgs, float*);
 enum KernelKind {
-  kKindPacked = 0, kKindScalar = 1, kKindSplit = 2, kKindGrad = 3, kKindShort = 6
+  kKindPacked = 0, kKindScalar = 1, kKindSplit = 2, kKindGrad = 3, kKindGradSplit = 4,
+  kKindGradAhead = 5, kKindShort = 6
 };
 
 template <int OP, int W, typename T, bool MV>
@@ -1042,7 +1361,9 @@ KFn pick_kind(int kind) {
     case kKindScalar: return k_semblance_scalar<OP, W, T, MV>;
     case kKindSplit: return k_semblance_split<OP, W, T, MV>;
     case kKindShort: return k_semblance_short<OP, W, T, MV>;
-    case kKindGrad: return k_semblance_grad<OP, W, T, MV>;
+    case kKindGrad: return k_semblance_grad<OP, W, T, MV, 1>;
+    case kKindGradAhead: return k_semblance_grad<OP, W, T, MV, 6>;
+    case kKindGradSplit: return k_semblance_grad_split<OP, W, T, MV>;
   }
   return nullptr;
 }

@@ -82,3 +82,35 @@ def test_slices_walked_by_one_warp_or_eight(op, w, storage, ns, sizes):
     if storage == "f32":
         ref = oracle.semblance.semblance_many(x, mid, off, prob, th[:, :2].cpu().numpy())
         assert np.max(np.abs(a[:, :2].cpu().numpy() - ref)) <= 1e-5
+
+
+@pytest.mark.parametrize("n_dom,P,sizes,op,w,storage,ns", [
+    (1, 1, (16,), 1, 5, "f32", 300), (63, 1, (64, 40), 1, 0, "f32", 300),
+    (65, 1, (300,), 2, 8, "f32", 300), (130, 3, (300, 17), 1, 8, "bf16", 300),
+    (500, 1, (257,), 1, 5, "f32", 2200), (40, 2, (70, 1, 33), 2, 1, "bf16", 2200),
+    (9000, 1, (300, 280), 1, 3, "f32", 300)])
+def test_split_gradient(n_dom, P, sizes, op, w, storage, ns):
+    """The split gradient (clusters of 1 to 8 blocks) against the unsplit one.
+    Both sum the same n = N (2w + 1) FP32 terms in different orders: S to
+    1e-6, as elsewhere between two orders. A gradient's terms cancel to about
+    1/sqrt(n) of their sum of magnitudes, so an error of at most n 2^-24 of
+    that sum is n^1.5 2^-24 of a typical gradient: 2.2e-2 for the longest
+    windows here (n = 5100), and 1/sqrt(n) of that, 3e-4, when roundings are
+    random; 1e-3 of |G| plus the median magnitude is asked."""
+    x, mid, off = _line(60, ns)
+    prob = _problem(n_dom, sizes, 60, ns, op, w)
+    th = to_dev(random_theta(n_dom, P, *BOUNDS[op], 5))
+    ctx = tt.tt_ctx_create(x, mid, off, prob, None, storage=storage, device=dev())
+    S, G = tt.tt_semblance_grad(ctx, th)
+    again = tt.tt_semblance_grad(ctx, th)
+    tt.tt_ctx_set_option(ctx, "split", False)
+    S0, G0 = tt.tt_semblance_grad(ctx, th)
+    ctx.close()
+    assert torch.equal(S, again[0]) and torch.equal(G, again[1])
+    assert (S - S0).abs().max().item() <= 1e-6
+    scale = G0.abs().flatten(0, 1).median(0).values
+    assert ((G - G0).abs() <= 1e-3 * (G0.abs() + scale)).all()
+    if storage == "f32":
+        rS, _ = oracle.semblance.semblance_grad_many(x, mid, off, prob, th.cpu().numpy()) \
+            if n_dom <= 500 else (None, None)
+        assert rS is None or np.max(np.abs(S.cpu().numpy() - rS)) <= 1e-5
