@@ -338,7 +338,9 @@ tt_status tt_ctx_probe_l1(tt_ctx* ctx, int32_t iters, double* bytes, void* strea
  *                 slice order; every variant then sums alike, so S
  *                 still does not depend on TT_OPT_KERNEL / TT_OPT_BLOCK, but
  *                 its rounding differs from the unsplit kernels' (all stay
- *                 within 1e-5 of the exact semblance). Gradient evaluations are
+ *                 within 1e-5 of the exact semblance). Searches of few domains
+ *                 with short apertures run all generations between exchanges
+ *                 in one launch, with the same sums. Gradient evaluations are
  *                 split too (tt_semblance_grad; not inside the polish, whose
  *                 iterates are compared by their S). 0: never split.
  *  TT_OPT_MEMBER_ORDER  1: before each generation's evaluation inside

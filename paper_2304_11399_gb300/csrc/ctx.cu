@@ -202,6 +202,15 @@ cudaError_t tt_ctx::semblance(const tt::EvalArgs& a, cudaStream_t s, bool grad) 
   return e;
 }
 
+cudaError_t tt_ctx::fused(const tt::EvalArgs& a, const tt::DeArgs& de, const tt::FusedArgs& f,
+                          cudaStream_t s) {
+  const int n = f.first ? f.last - f.first + 1 : f.last + 1;
+  ++n_launch;
+  n_sem += n;
+  trace_evals += double(a.P) * sum_N * n;
+  return tt::launch_fused_search(a, de, f, s);
+}
+
 extern "C" tt_status tt_ctx_profile(tt_ctx* c, int32_t enable) {
   if (!c) return tt_fail(nullptr, TT_ERR_INVALID_ARG, "ctx is NULL");
   if (enable && c->ev.empty()) {

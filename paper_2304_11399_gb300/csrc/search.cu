@@ -115,73 +115,100 @@ tt_status search_body(tt_ctx* c, float* best_theta, float* best_S, cudaStream_t 
     ea.np_out = NP;
     return tt_cuda_check(c, c->semblance(ea, s, false), "evaluate");
   };
-  // generation 0: initialise and evaluate
-  tt::DeArgs a = de_args(0);
-  a.pop = c->pop;
-  a.fit = c->fit;
-  STEP(c->counted(tt::launch_de_step(a, s)), "init");
-  st = evaluate(c->pop, c->fit, c->trial[0], c->tfit[0]);
-  if (st != TT_OK) return st;
-  evals += (unsigned long long)NP * c->n_dom;
-  int cur = 0;            // trial buffer written by the next mutation
-  bool pending = false;   // trial[cur ^ 1] awaits selection
-  for (int g = 1; g <= NG; ++g) {
-    a = de_args(g);
+  // the neighbour exchange after the selection of generation g
+  auto exchange = [&](int g) -> tt_status {
+    STEP(c->counted(tt::launch_best_snapshot(c->n_dom, NP, c->D, c->pop, c->fit, c->snap,
+                                              nullptr, s)),
+         "snapshot");
+    if (prev || next) {
+      // the edge rows out, the neighbouring slabs' rows in
+      const size_t row = size_t(c->n_t0) * c->D * sizeof(float);
+      STEP(cudaMemcpyAsync(slab->send_first, c->snap, row, cudaMemcpyDeviceToDevice, s),
+           "send first row");
+      STEP(cudaMemcpyAsync(slab->send_last, c->snap + size_t(c->n_m0 - 1) * c->n_t0 * c->D,
+                           row, cudaMemcpyDeviceToDevice, s),
+           "send last row");
+      if (slab->exchange(slab->user, g, s) != 0)
+        return tt_fail(c, TT_ERR_INVALID_ARG, "slab exchange callback failed at gen %d", g);
+    }
+    STEP(c->counted(tt::launch_exchange_plan(c->n_m0, c->n_t0, NP, c->D, c->snap, c->pop,
+                                             c->fit, c->imports, c->slots, s,
+                                             prev ? slab->recv_prev : nullptr,
+                                             next ? slab->recv_next : nullptr)),
+         "exchange");
+    tt::EvalArgs ea = c->eval_args(c->imports, 4, c->fit);
+    ea.slots = c->slots;
+    ea.np_out = NP;
+    STEP(c->semblance(ea, s, false), "evaluate imports");
+    return TT_OK;
+  };
+  tt::EvalArgs whole = c->eval_args(c->pop, NP, c->fit);
+  if (!c->profiling && c->member_order != 1 && tt::fused_search_fits(whole)) {
+    // all generations up to the next exchange in one launch
+    for (int g = 0; g <= NG;) {
+      const bool ex = grid && (g ? g : 1) <= NG - NG % cfg.exch_every;
+      const int from = g ? g : 1;
+      const int to = ex ? (from + cfg.exch_every - 1) / cfg.exch_every * cfg.exch_every : NG;
+      tt::DeArgs d = de_args(0);
+      d.pop = c->pop;
+      d.fit = c->fit;
+      STEP(c->fused(whole, d, tt::FusedArgs{g, to}, s), "generations");
+      if (ex) {
+        st = exchange(to);
+        if (st != TT_OK) return st;
+        evals += edges;
+      }
+      g = to + 1;
+    }
+    evals += (unsigned long long)NP * c->n_dom * (NG + 1);
+  } else {
+    // generation 0: initialise and evaluate
+    tt::DeArgs a = de_args(0);
     a.pop = c->pop;
     a.fit = c->fit;
-    a.trial = pending ? c->trial[cur ^ 1] : nullptr;
-    a.tfit = pending ? c->tfit[cur ^ 1] : nullptr;
-    a.next = c->trial[cur];
-    STEP(c->counted(tt::launch_de_step(a, s)), "de step");
-    // the selection above has consumed trial[cur ^ 1]: free for the reordered copy
-    st = evaluate(c->trial[cur], c->tfit[cur], c->trial[cur ^ 1], c->tfit[cur ^ 1]);
+    STEP(c->counted(tt::launch_de_step(a, s)), "init");
+    st = evaluate(c->pop, c->fit, c->trial[0], c->tfit[0]);
     if (st != TT_OK) return st;
     evals += (unsigned long long)NP * c->n_dom;
-    pending = true;
-    cur ^= 1;
-    if (grid && g % cfg.exch_every == 0) {
+    int cur = 0;            // trial buffer written by the next mutation
+    bool pending = false;   // trial[cur ^ 1] awaits selection
+    for (int g = 1; g <= NG; ++g) {
       a = de_args(g);
-      a.sel_gen = g;  // select-only: the trial of this generation
+      a.pop = c->pop;
+      a.fit = c->fit;
+      a.trial = pending ? c->trial[cur ^ 1] : nullptr;
+      a.tfit = pending ? c->tfit[cur ^ 1] : nullptr;
+      a.next = c->trial[cur];
+      STEP(c->counted(tt::launch_de_step(a, s)), "de step");
+      // the selection above has consumed trial[cur ^ 1]: free for the reordered copy
+      st = evaluate(c->trial[cur], c->tfit[cur], c->trial[cur ^ 1], c->tfit[cur ^ 1]);
+      if (st != TT_OK) return st;
+      evals += (unsigned long long)NP * c->n_dom;
+      pending = true;
+      cur ^= 1;
+      if (grid && g % cfg.exch_every == 0) {
+        a = de_args(g);
+        a.sel_gen = g;  // select-only: the trial of this generation
+        a.pop = c->pop;
+        a.fit = c->fit;
+        a.trial = c->trial[cur ^ 1];
+        a.tfit = c->tfit[cur ^ 1];
+        STEP(c->counted(tt::launch_de_step(a, s)), "select");
+        pending = false;
+        st = exchange(g);
+        if (st != TT_OK) return st;
+        evals += edges;
+      }
+    }
+    if (pending) {
+      a = de_args(NG + 1);
+      a.sel_gen = NG;  // select-only: the last trial
       a.pop = c->pop;
       a.fit = c->fit;
       a.trial = c->trial[cur ^ 1];
       a.tfit = c->tfit[cur ^ 1];
-      STEP(c->counted(tt::launch_de_step(a, s)), "select");
-      pending = false;
-      STEP(c->counted(tt::launch_best_snapshot(c->n_dom, NP, c->D, c->pop, c->fit, c->snap,
-                                                nullptr, s)),
-           "snapshot");
-      if (prev || next) {
-        // the edge rows out, the neighbouring slabs' rows in
-        const size_t row = size_t(c->n_t0) * c->D * sizeof(float);
-        STEP(cudaMemcpyAsync(slab->send_first, c->snap, row, cudaMemcpyDeviceToDevice, s),
-             "send first row");
-        STEP(cudaMemcpyAsync(slab->send_last, c->snap + size_t(c->n_m0 - 1) * c->n_t0 * c->D,
-                             row, cudaMemcpyDeviceToDevice, s),
-             "send last row");
-        if (slab->exchange(slab->user, g, s) != 0)
-          return tt_fail(c, TT_ERR_INVALID_ARG, "slab exchange callback failed at gen %d", g);
-      }
-      STEP(c->counted(tt::launch_exchange_plan(c->n_m0, c->n_t0, NP, c->D, c->snap, c->pop,
-                                               c->fit, c->imports, c->slots, s,
-                                               prev ? slab->recv_prev : nullptr,
-                                               next ? slab->recv_next : nullptr)),
-           "exchange");
-      tt::EvalArgs ea = c->eval_args(c->imports, 4, c->fit);
-      ea.slots = c->slots;
-      ea.np_out = NP;
-      STEP(c->semblance(ea, s, false), "evaluate imports");
-      evals += edges;
+      STEP(c->counted(tt::launch_de_step(a, s)), "final select");
     }
-  }
-  if (pending) {
-    a = de_args(NG + 1);
-    a.sel_gen = NG;  // select-only: the last trial
-    a.pop = c->pop;
-    a.fit = c->fit;
-    a.trial = c->trial[cur ^ 1];
-    a.tfit = c->tfit[cur ^ 1];
-    STEP(c->counted(tt::launch_de_step(a, s)), "final select");
   }
   STEP(c->counted(tt::launch_best_snapshot(c->n_dom, NP, c->D, c->pop, c->fit, best_theta,
                                            best_S, s)),

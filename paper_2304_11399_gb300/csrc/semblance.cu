@@ -14,6 +14,9 @@ extern template SFn pick_stack<TT_OP_FOCRS>(int, bool, int);
 extern template OFn pick_order<TT_OP_CMP>(bool);
 extern template OFn pick_order<TT_OP_CRS>(bool);
 extern template OFn pick_order<TT_OP_FOCRS>(bool);
+extern template FFn pick_fused<TT_OP_CMP>(int, int, bool);
+extern template FFn pick_fused<TT_OP_CRS>(int, int, bool);
+extern template FFn pick_fused<TT_OP_FOCRS>(int, int, bool);
 }  // namespace sk
 
 namespace {
@@ -204,6 +207,39 @@ cudaError_t launch_stack(const EvalArgs& a, float* out, cudaStream_t s) {
 }
 
 cudaError_t launch_semblance_grad(const EvalArgs& a, cudaStream_t s) { return launch(a, s, true); }
+
+// Apertures of up to 160 traces, or of 1.5 per unit where the 64 slots of a
+// block are nearly full: DE 32 x 30 on 38 / 150 / 300 units of 48 traces 144 /
+// 134 / 173 us against 291 / 302 / 344 us stepwise, of 144 traces 253 / 267 /
+// 370 against 289 / 504 / 525, of 336 traces 446 / 665 / 799 against 341 / 672
+// / 1122, of 1008 traces 1258 / 1898 / 2164 against 602 / 1352 / 2297.
+bool fused_search_fits(const EvalArgs& a) {
+  const long long units = ((long long)a.n_dom * a.P + 63) / 64;
+  if (!a.split || a.P > 64 || a.dom_map || units > (long long)a.n_sm * kSplitSmallPerSm)
+    return false;
+  return a.mean_ap <= 160.f ||
+         (a.mean_ap <= 1.5f * float(units) && 64 / a.P * a.P * 6 >= 64 * 5);
+}
+
+cudaError_t launch_fused_search(const EvalArgs& a, const DeArgs& de, const FusedArgs& f,
+                                cudaStream_t s) {
+  if (a.n_dom == 0) return cudaSuccess;
+  const bool mv = a.umax > float(kDirectMax);
+  sk::FFn fn = nullptr;
+  switch (a.op) {
+    case TT_OP_CMP: fn = sk::pick_fused<TT_OP_CMP>(a.storage, a.W, mv); break;
+    case TT_OP_CRS: fn = sk::pick_fused<TT_OP_CRS>(a.storage, a.W, mv); break;
+    case TT_OP_FOCRS: fn = sk::pick_fused<TT_OP_FOCRS>(a.storage, a.W, mv); break;
+  }
+  if (!fn || a.P > 64) return cudaErrorInvalidValue;
+  const int B = split_blocks(((long long)a.n_dom * a.P + 63) / 64, a.n_sm);
+  const int per = 64 / a.P;
+  const size_t smem = sk::short_smem_bytes(B, a.W, a.storage == TT_STORE_BF16);
+  const cudaError_t e = allow_smem(fn, smem);
+  if (e != cudaSuccess) return e;
+  fn<<<(a.n_dom + per - 1) / per, 32 * B, smem, s>>>(a, de, f);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_member_order(const EvalArgs& a, float* theta_out, int* slots,
                                 cudaStream_t s) {

@@ -39,6 +39,7 @@
 
 #include <cooperative_groups.h>
 
+#include "de_kernels.cuh"
 #include "tt_internal.cuh"
 
 namespace tt {
@@ -107,19 +108,9 @@ __device__ __forceinline__ int dom_of(long long q, int P) {
 
 // L.d is the local domain (indexing theta and S); its geometry comes from the
 // global domain dom_map[L.d] when a map is given (a subset evaluation).
-template <int OP, bool DIV32 = false>
-__device__ __forceinline__ bool lane_setup(const EvalArgs& a, long long q, Lane& L) {
-  if (q >= (long long)a.n_dom * a.P) return false;
-  L.d = DIV32 ? dom_of(q, a.P) : int(q / a.P);
-  const int gd = a.dom_map ? a.dom_map[L.d] : L.d;
-  if (gd < 0) return false;
-  const int g = a.dom_group[gd];
-  L.inv_dt = a.g_inv_dt[g];
-  L.e0 = a.ap_ptr[g];
-  L.e1 = a.ap_ptr[g + 1];
-  L.p0i = a.dom_it0[gd];
-  L.p0 = float(L.p0i);
-  const float* th = a.theta + q * op_dim(OP);
+// The operator's coefficients of parameter vector th in sample units.
+template <int OP>
+__device__ __forceinline__ void set_theta(Lane& L, const float* th) {
   const float i2 = L.inv_dt * L.inv_dt;
   L.cah = 0.f;
   L.cbh = 0.f;
@@ -138,6 +129,22 @@ __device__ __forceinline__ bool lane_setup(const EvalArgs& a, long long q, Lane&
     L.cbh = th[3] * i2;
     L.cc = th[4] * i2;
   }
+}
+
+template <int OP, bool DIV32 = false>
+__device__ __forceinline__ bool lane_setup(const EvalArgs& a, long long q, Lane& L) {
+  if (q >= (long long)a.n_dom * a.P) return false;
+  L.d = DIV32 ? dom_of(q, a.P) : int(q / a.P);
+  const int gd = a.dom_map ? a.dom_map[L.d] : L.d;
+  if (gd < 0) return false;
+  const int g = a.dom_group[gd];
+  L.inv_dt = a.g_inv_dt[g];
+  L.e0 = a.ap_ptr[g];
+  L.e1 = a.ap_ptr[g + 1];
+  L.p0i = a.dom_it0[gd];
+  L.p0 = float(L.p0i);
+  const float* th = a.theta + q * op_dim(OP);
+  set_theta<OP>(L, th);
   L.two_p0 = 2.f * L.p0;
   L.p0sq = __fmul_rn(L.p0, L.p0) + 1e-30f;
   L.lim = a.umax - L.p0;
@@ -437,7 +444,7 @@ __device__ __forceinline__ void eval_unit(const EvalArgs& a, long long unit, int
 // 1824 units on a 152-SM device). The summation order depends on B and differs
 // from the one-warp-per-unit kernel, so B is chosen by launch size alone --
 // every variant of a launch gives the same bits -- and results stay
-// reproducible. Two kernels run it, with the same bits:
+// reproducible. Three kernels run it, with the same bits:
 //  * k_semblance_split: a warp per slice, eight warps per block, a cluster of
 //    B blocks per unit. The blocks push their sums into the first one's shared
 //    memory and leave; no global scratch, fence, ticket or re-read. Latency
@@ -447,6 +454,7 @@ __device__ __forceinline__ void eval_unit(const EvalArgs& a, long long unit, int
 //  * k_semblance_short: a warp per eight slices, walked one after the other,
 //    for apertures too short to feed 8 B warps (258 units x 48 traces: 10.4 us
 //    against 18.5 us with a warp per slice and 29.1 us through scratch).
+//  * k_search_short: the same walk inside a whole search.
 constexpr int kSplitWarps = 8;
 
 // Slice sl of nsl of a pair's aperture: entries floor(n sl / nsl) to
@@ -477,7 +485,7 @@ inline size_t split_smem_bytes(int B, int W, bool bf16) {
   const size_t set = bf16 ? split_set_bytes<__nv_bfloat16>(W) : split_set_bytes<float>(W);
   return set * size_t(kSplitWarps + (B > 1 ? B : 0));
 }
-// k_semblance_short: the unit's B sums
+// k_semblance_short and k_search_short: the unit's B sums
 inline size_t short_smem_bytes(int B, int W, bool bf16) {
   const size_t set = bf16 ? split_set_bytes<__nv_bfloat16>(W) : split_set_bytes<float>(W);
   return set * size_t(B);
@@ -784,6 +792,102 @@ __global__ void __launch_bounds__(32 * kSplitSmallBlocks, 2) k_semblance_short(c
   if (Chunk<T>::kF64)
     for (int c = 0; c < B; ++c) Ed += set_Ed[c * 64 + p];
   finish_pair<W, T>(a, unit * 64 + p, size[p], set + p, Ed);
+}
+
+// The search of short apertures and few domains, generation after generation
+// in one launch: nothing but the neighbour exchange couples domains, so a block
+// of B warps takes the 64 / NP domains of a unit and runs evaluation and DE
+// step in turn on populations that stay in shared memory. A generation of such
+// a search is a few microseconds of dependent work; as two launches it costs
+// as much again in launch latency, and each kernel reads what the one before
+// wrote from L2. Each pair's semblance is that of the stepwise search bit for
+// bit: the same 8 B slices of its aperture, B by the size of the stepwise
+// launch; so are the DE steps (de_kernels.cuh). Bound by the latency of the
+// seven warps' instructions (about 6,000 of a generation's 9,000 cycles are
+// the evaluation). 128 registers, so that two blocks fit an SM: 500 CMP
+// domains x 48 traces, DE 32 x 50: 239 us, against 526 us stepwise with
+// k_semblance_short and 1,525 us before that.
+template <int OP, int W, typename T, bool MV>
+__global__ void __maxnreg__(128)
+    k_search_short(const EvalArgs a, const DeArgs de, const FusedArgs fa) {
+  constexpr int K = 2 * W + 1, R = K + 1;
+  constexpr int D = op_dim(OP);
+  extern __shared__ __align__(16) unsigned char split_smem[];
+  __shared__ float pop[64 * D], trial[64 * D], fit[64], tfit[64];
+  __shared__ int size[64];
+  const int B = blockDim.x >> 5, nt = blockDim.x, NP = a.P;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double* set_Ed = reinterpret_cast<double*>(split_smem);  // [B][64]
+  float* set = reinterpret_cast<float*>(set_Ed + (Chunk<T>::kF64 ? B * 64 : 0));
+  const int per = 64 / NP, dom0 = blockIdx.x * per;  // the block's domains
+  const int nd = min(per, a.n_dom - dom0), n = nd * NP;  // and pairs
+  // a lane without a second pair walks its first one twice
+  const bool v0 = lane < n, v1 = lane + 32 < n;
+  const int p1 = v1 ? lane + 32 : lane;
+  Lane L0, L1;
+  lane_setup<OP, true>(a, (long long)dom0 * NP + (v0 ? lane : 0), L0);
+  lane_setup<OP, true>(a, (long long)dom0 * NP + (v0 ? p1 : 0), L1);
+  if (w == 0) keep_sizes(size, lane, v0, L0, v1, L1);
+  Slices A0, A1;
+  A0.set(L0, kSplitWarps * B, kSplitWarps * w);
+  A1.set(L1, kSplitWarps * B, kSplitWarps * w);
+  auto evaluate = [&](const float* th, float* S) {
+    if (v0) {
+      set_theta<OP>(L0, th + lane * D);
+      set_theta<OP>(L1, th + p1 * D);
+    }
+    unit_slices<OP, W, T, MV>(a, v0, L0, A0, v0, L1, A1, lane, set + w * R * 64, set_Ed + w * 64);
+    __syncthreads();
+    if (B == kSplitSmallBlocks)
+      add_sets<W, kSplitSmallBlocks>(set, threadIdx.x);
+    else
+      add_sets<W, kSplitTinyBlocks>(set, threadIdx.x);
+    __syncthreads();
+    if (threadIdx.x < n) {
+      const int p = threadIdx.x;
+      double Ed = 0.0;
+      if (Chunk<T>::kF64)
+        for (int c = 0; c < B; ++c) Ed += set_Ed[c * 64 + p];
+      float Q = 0.f;
+#pragma unroll
+      for (int k = 0; k < K; ++k) Q = fmaf(set[k * 64 + p], set[k * 64 + p], Q);
+      S[p] = normalise<T>(Q, size[p], set[K * 64 + p], Ed);
+    }
+    __syncthreads();
+  };
+  auto step = [&](int gen, int sel_gen, bool select, bool mutate) {
+    for (int i = w; i < nd; i += B) {
+      const int o = i * NP;
+      de::DePop p;
+      p.pop = p.spop = pop + o * D;
+      p.fit = p.sfit = fit + o;
+      p.trial = select ? trial + o * D : nullptr;
+      p.tfit = tfit + o;
+      p.next = mutate ? trial + o * D : nullptr;
+      de::de_step<D>(de, dom0 + i, uint32_t(de.dom_base + dom0 + i), uint32_t(gen),
+                     uint32_t(sel_gen), p, lane);
+    }
+    __syncthreads();
+  };
+  const size_t row = (size_t)dom0 * NP;
+  if (fa.first == 0) {
+    for (int i = w; i < nd; i += B)
+      de::de_init<D>(de, dom0 + i, uint32_t(de.dom_base + dom0 + i), pop + i * NP * D, lane);
+    __syncthreads();
+    evaluate(pop, fit);
+  } else {
+    for (int i = threadIdx.x; i < n * D; i += nt) pop[i] = de.pop[row * D + i];
+    for (int i = threadIdx.x; i < n; i += nt) fit[i] = de.fit[row + i];
+    __syncthreads();
+  }
+  const int g0 = fa.first ? fa.first : 1;
+  for (int g = g0; g <= fa.last; ++g) {
+    step(g, g - 1, g > g0, true);
+    evaluate(trial, tfit);
+  }
+  if (fa.last >= g0) step(fa.last + 1, fa.last, true, false);
+  for (int i = threadIdx.x; i < n * D; i += nt) de.pop[row * D + i] = pop[i];
+  for (int i = threadIdx.x; i < n; i += nt) de.fit[row + i] = fit[i];
 }
 
 // K1, grid-mapped (queue == nullptr: one 64-pair unit per warp, the grid
@@ -1339,6 +1443,32 @@ __global__ void __launch_bounds__(32 * kOrderWarps) k_member_order(const EvalArg
     for (int k = 0; k < D; ++k) dst[k] = src[k];
     slots[d * P + rank] = i;
   }
+}
+
+using FFn = void (*)(const EvalArgs, const DeArgs, const FusedArgs);
+
+template <int OP, typename T, bool MV>
+FFn pick_fused_w(int W) {
+  switch (W) {
+    case 0: return k_search_short<OP, 0, T, MV>;
+    case 1: return k_search_short<OP, 1, T, MV>;
+    case 2: return k_search_short<OP, 2, T, MV>;
+    case 3: return k_search_short<OP, 3, T, MV>;
+    case 4: return k_search_short<OP, 4, T, MV>;
+    case 5: return k_search_short<OP, 5, T, MV>;
+    case 6: return k_search_short<OP, 6, T, MV>;
+    case 7: return k_search_short<OP, 7, T, MV>;
+    case 8: return k_search_short<OP, 8, T, MV>;
+  }
+  return nullptr;
+}
+
+template <int OP>
+FFn pick_fused(int storage, int W, bool mv) {
+  const bool bf = storage == TT_STORE_BF16;
+  if (mv)
+    return bf ? pick_fused_w<OP, __nv_bfloat16, true>(W) : pick_fused_w<OP, float, true>(W);
+  return bf ? pick_fused_w<OP, __nv_bfloat16, false>(W) : pick_fused_w<OP, float, false>(W);
 }
 
 using OFn = void (*)(const EvalArgs, float*, int*);

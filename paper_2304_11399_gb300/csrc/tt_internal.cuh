@@ -108,6 +108,17 @@ struct DeArgs {
 
 cudaError_t launch_de_step(const DeArgs& a, cudaStream_t s);
 
+// Generations of a fused search launch: from `first` (0: initialise and
+// evaluate generation 0, then from 1 on) to the selection of `last`.
+struct FusedArgs {
+  int first, last;
+};
+// Whether a search of this population takes the fused form, and its launch
+// (pop and fit of de hold the populations between launches).
+bool fused_search_fits(const EvalArgs& a);
+cudaError_t launch_fused_search(const EvalArgs& a, const DeArgs& de, const FusedArgs& f,
+                                cudaStream_t s);
+
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): 10 rounds of
 // (c0, c1, c2, c3) -> (hi(M1 c2) ^ c1 ^ k0, lo(M1 c2), hi(M0 c0) ^ c3 ^ k1,
 // lo(M0 c0)), key bumped by the Weyl constants between rounds.
@@ -245,6 +256,9 @@ struct tt_ctx {
   tt::EvalArgs eval_args(const float* theta, int P, float* S) const;
   // every semblance / gradient launch of the library goes through here
   cudaError_t semblance(const tt::EvalArgs& a, cudaStream_t s, bool grad);
+  // a fused search launch, counted as the evaluations it holds
+  cudaError_t fused(const tt::EvalArgs& a, const tt::DeArgs& de, const tt::FusedArgs& f,
+                    cudaStream_t s);
   cudaError_t counted(cudaError_t e) {
     ++n_launch;
     return e;

@@ -114,3 +114,43 @@ def test_split_gradient(n_dom, P, sizes, op, w, storage, ns):
         rS, _ = oracle.semblance.semblance_grad_many(x, mid, off, prob, th.cpu().numpy()) \
             if n_dom <= 500 else (None, None)
         assert rS is None or np.max(np.abs(S.cpu().numpy() - rS)) <= 1e-5
+
+
+def _cfg(op, np_, ng, **kw):
+    kw = {"exch_every": 0, "polish_steps": 0, "polish_lr": 2e-4, "adapt": 0, **kw}
+    lo, hi = BOUNDS[op]
+    return configs.DEConfig(np=np_, ng=ng, F=0.5, CR=0.9, seed=11, lo=lo, hi=hi, **kw)
+
+
+@pytest.mark.parametrize("n_dom,np_,ng,op,w,storage,ns,sizes,kw", [
+    (1, 4, 3, 1, 5, "f32", 300, (40,), {}), (37, 64, 0, 1, 5, "f32", 300, (40, 57), {}),
+    (65, 37, 5, 2, 8, "bf16", 300, (70, 0, 33), {"adapt": 1}),
+    (300, 13, 7, 1, 0, "f32", 2200, (150,), {"adapt": 1}),
+    (297, 64, 4, 1, 5, "bf16", 300, (56, 1, 120), {}),
+    (600, 30, 9, 1, 5, "f32", 300, (60, 20), {"grid": (20, 30), "exch_every": 3, "polish_steps": 2}),
+    (60, 9, 8, 1, 2, "f32", 300, (30,), {"grid": (6, 10), "exch_every": 5, "adapt": 1})])
+def test_fused_search_equals_stepwise(n_dom, np_, ng, op, w, storage, ns, sizes, kw):
+    """All generations between exchanges in one launch against one launch per
+    step (what a search runs while its launches are timed): the same bits."""
+    kw = dict(kw)
+    grid = kw.pop("grid", None)
+    x, mid, off = _line(60, ns)
+    prob = _problem(n_dom, sizes, 60, ns, op, w)
+    if grid:
+        prob.n_m0, prob.n_t0 = grid
+    ctx = tt.tt_ctx_create(x, mid, off, prob, _cfg(op, np_, ng, **kw), storage=storage,
+                           device=dev())
+    th, S, n = tt.tt_search(ctx)
+    tt.tt_ctx_set_option(ctx, "search_graph", False)
+    tt.tt_ctx_stats(ctx, reset=True)
+    th1, S1, n1 = tt.tt_search(ctx)
+    few = tt.tt_ctx_stats(ctx, reset=True)
+    tt.tt_ctx_profile(ctx, True)
+    th2, S2, n2 = tt.tt_search(ctx)
+    many = tt.tt_ctx_stats(ctx)
+    ctx.close()
+    assert torch.equal(th, th2) and torch.equal(S, S2) and n == n2
+    assert torch.equal(th, th1) and torch.equal(S, S1) and n == n1
+    assert few["launches"] < many["launches"] or ng == 0
+    assert few["trace_evals"] == many["trace_evals"]
+    assert few["semblance_launches"] == many["semblance_launches"]
