@@ -323,7 +323,7 @@ tt_status tt_ctx_probe_l1(tt_ctx* ctx, int32_t iters, double* bytes, void* strea
  *                 uneven apertures), TT_KERNEL_SCALAR (one pair per thread).
  *                 All variants perform the same operations in the same order
  *                 and give bit-identical S.
- *  TT_OPT_BLOCK   threads per block, 128 or 256 (default 256).
+ *  TT_OPT_BLOCK   threads per block, 128 or 256 (default 128).
  *  TT_OPT_SEARCH_GRAPH  1 (default): tt_search captures its whole launch
  *                 sequence into a CUDA graph on first use and replays it;
  *                 0: launch eagerly. Searches run eagerly while profiling is

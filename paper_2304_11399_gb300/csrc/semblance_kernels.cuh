@@ -890,12 +890,23 @@ __global__ void __maxnreg__(128)
   for (int i = threadIdx.x; i < n; i += nt) de.fit[row + i] = fit[i];
 }
 
+// Blocks of kBlock threads that K1 asks the compiler to fit on an SM: 4 (64
+// registers) for FO-CRS and for BF16 storage at windows up to 11 samples, where
+// the compiler left to itself takes 72 and more (w = 5, 128-thread blocks:
+// FO-CRS 18,000 domains x 64 2.09 -> 1.93 ms, moveout form 3.78 -> 3.60 ms, BF16
+// moveout form 5.83 -> 5.53 ms); 0, no request, for the others (asking for 4
+// costs the FP32 CRS direct form, at 64 registers either way, 1.4%).
+template <int OP, int W, typename T>
+constexpr int k1_blocks() {
+  return W <= 5 && (OP == TT_OP_FOCRS || sizeof(T) == 2) ? 4 : 0;
+}
+
 // K1, grid-mapped (queue == nullptr: one 64-pair unit per warp, the grid
 // covers every unit) or persistent (a grid sized to the GPU; after its first
 // unit a warp takes the next one from an atomic counter, so warps whose
 // apertures are short take more units).
 template <int OP, int W, typename T, bool MV>
-__global__ void __launch_bounds__(kBlock) k_semblance(const EvalArgs a) {
+__global__ void __launch_bounds__(kBlock, k1_blocks<OP, W, T>()) k_semblance(const EvalArgs a) {
   const int lane = threadIdx.x & 31;
   const long long n_units = ((long long)a.n_dom * a.P + 63) / 64;
   const long long warps = (long long)gridDim.x * (blockDim.x >> 5);

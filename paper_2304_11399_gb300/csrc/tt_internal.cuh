@@ -229,7 +229,11 @@ struct tt_ctx {
   cudaStream_t side_stream = nullptr;
   cudaEvent_t side_ev[4] = {nullptr, nullptr, nullptr, nullptr};
   // launch configuration (tt_ctx_set_option / tt_ctx_autotune)
-  int kernel = TT_KERNEL_PACKED, block = 256;
+  // 128 threads per block by default: slots are refilled four warps at a time
+  // instead of eight, and the moveout form's 72 registers leave room for 28
+  // warps per SM instead of 24 (CRS line 20 CMPs x 64 random 5.42 -> 5.34 ms,
+  // converged 4.31 -> 4.24 ms; 64 uneven problems, moveout form, 3.30 -> 2.98 ms)
+  int kernel = TT_KERNEL_PACKED, block = 128;
   bool split = true;  // TT_OPT_SPLIT
   int member_order = 2;  // TT_OPT_MEMBER_ORDER: 0 index order, 1 member order, 2 automatic
   bool use_graph = true;
