@@ -88,28 +88,31 @@ cudaError_t launch_split(EvalArgs& a, long long units, bool mv, cudaStream_t s) 
   return cudaLaunchKernelEx(&cfg, fn, a);
 }
 
-// Split gradient launches: with apertures of 256 traces or more at every size
-// (1008 traces: 24 / 938 / 9375 units 28 / 474 / 3763 us against 740 / 839 /
-// 4101 us with one pair per thread), with shorter ones down to 16 traces while
-// the launch has fewer than 16 units per SM (144 traces: 469 units 75 us
-// against 98 us, 4688 units 322 us against 307 us; 48 traces: 16 units 18 us
-// against 50 us, 9375 units 284 us against 217 us).
+// Split gradient launches: where forward launches split (their sums then agree
+// bit for bit, and so does S), with apertures of 256 traces or more (1008
+// traces: 24 / 938 / 4688 units 28 / 474 / 1963 us against 740 / 839 / 2126 us
+// with one pair per thread), with shorter ones down to 16 traces while the
+// launch has fewer than 16 units per SM (144 traces: 469 units 75 us against
+// 98 us, 4688 units 322 us against 307 us; 48 traces: 16 units 18 us against 50
+// us, 9375 units 284 us against 217 us).
 bool grad_split(const EvalArgs& a, long long units) {
-  return a.split && (a.mean_ap >= 256.f || (a.mean_ap >= 16.f && units < 16ll * a.n_sm));
+  return a.split && units < (long long)a.n_sm * kSplitUnitsPerSm &&
+         (a.mean_ap >= 256.f || (a.mean_ap >= 16.f && units < 16ll * a.n_sm));
 }
 
-// The cluster grows to 8 blocks while the launch has fewer than 7 blocks per SM
-// (three run on an SM at a time, so that the last wave weighs little) and the
-// slices hold 4 traces on average (1008 traces, clusters of 1 / 2 / 4 / 8: 24
-// units 115 / 66 / 38 / 28 us, 282 units 308 / 235 / 207 / 217 us, 938 units
-// 647 / 562 / 577 / 680 us, at two blocks per SM).
+// The cluster has the forward launch's B blocks (1008 traces, clusters of 1 / 2
+// / 4 / 8: 24 units 115 / 66 / 38 / 28 us, 282 units 308 / 235 / 207 / 217 us,
+// 938 units 647 / 562 / 577 / 680 us, at two blocks per SM: the rule's 9, 7 and
+// 2 lie near the best).
 cudaError_t launch_grad_split(const EvalArgs& a, long long units, bool mv, cudaStream_t s) {
   const KFn fn = pick(sk::kKindGradSplit, a, mv);
   if (!fn) return cudaErrorInvalidValue;
-  int B = 1;
-  while (B < sk::kGradMaxCluster && units * B < 7ll * a.n_sm &&
-         a.mean_ap >= float(4 * sk::kGradWarps * B))
-    B *= 2;
+  const int B = split_blocks(units, a.n_sm);
+  if (B > 8) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
   if (units * B > 0x7fffffffll) return cudaErrorInvalidConfiguration;
   cudaLaunchAttribute attr{};
   attr.id = cudaLaunchAttributeClusterDimension;

@@ -1164,7 +1164,6 @@ __global__ void __launch_bounds__(128) k_semblance_grad(const EvalArgs a) {
 // than two (102 registers: 562 us); it stays bound by its window loads (two
 // passes at K1's rate).
 constexpr int kGradWarps = 8;
-constexpr int kGradMaxCluster = 8;
 
 // shared memory of a block: FP64 energies [kGradWarps + 1][64]; rows of 64
 // floats that hold the slice sums of s and E [kGradWarps][K + 1], later the

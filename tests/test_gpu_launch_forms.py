@@ -88,9 +88,9 @@ def test_slices_walked_by_one_warp_or_eight(op, w, storage, ns, sizes):
     (1, 1, (16,), 1, 5, "f32", 300), (63, 1, (64, 40), 1, 0, "f32", 300),
     (65, 1, (300,), 2, 8, "f32", 300), (130, 3, (300, 17), 1, 8, "bf16", 300),
     (500, 1, (257,), 1, 5, "f32", 2200), (40, 2, (70, 1, 33), 2, 1, "bf16", 2200),
-    (9000, 1, (300, 280), 1, 3, "f32", 300)])
+    (9000, 1, (300, 280), 1, 3, "f32", 300), (25000, 1, (60,), 1, 5, "bf16", 300)])
 def test_split_gradient(n_dom, P, sizes, op, w, storage, ns):
-    """The split gradient (clusters of 1 to 8 blocks) against the unsplit one.
+    """The split gradient (clusters of 9, 7 and 2 blocks) against the unsplit one.
     Both sum the same n = N (2w + 1) FP32 terms in different orders: S to
     1e-6, as elsewhere between two orders. A gradient's terms cancel to about
     1/sqrt(n) of their sum of magnitudes, so an error of at most n 2^-24 of
@@ -103,6 +103,7 @@ def test_split_gradient(n_dom, P, sizes, op, w, storage, ns):
     ctx = tt.tt_ctx_create(x, mid, off, prob, None, storage=storage, device=dev())
     S, G = tt.tt_semblance_grad(ctx, th)
     again = tt.tt_semblance_grad(ctx, th)
+    assert torch.equal(S, tt.tt_semblance_eval(ctx, th))  # the forward's slices and order
     tt.tt_ctx_set_option(ctx, "split", False)
     S0, G0 = tt.tt_semblance_grad(ctx, th)
     ctx.close()
