@@ -74,17 +74,21 @@ cudaError_t launch_split(EvalArgs& a, long long units, bool mv, cudaStream_t s) 
   if (e == cudaSuccess && B > 8)  // more blocks than every device has to offer
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = unsigned(B);
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  // load-balancing rather than spread placement of the clusters: ENS 5 x 1 sweep
+  // 19.3 -> 18.6 ms, 125 units x 6120 traces 168 -> 160 us
+  cudaLaunchAttribute attr[2] = {};
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = unsigned(B);
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeClusterSchedulingPolicyPreference;
+  attr[1].val.clusterSchedulingPolicyPreference = cudaClusterSchedulingPolicyLoadBalancing;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(unsigned(units * B));
   cfg.blockDim = dim3(32 * sk::kSplitWarps);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, fn, a);
 }
 

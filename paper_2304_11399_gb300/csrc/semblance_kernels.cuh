@@ -480,10 +480,21 @@ constexpr size_t split_set_bytes(int W) {
   return 64 * (sizeof(float) * (2 * W + 2) + (Chunk<T>::kF64 ? sizeof(double) : 0));
 }
 // k_semblance_split: the block's eight slices, and (used by the cluster's
-// first block) the B blocks' sums
+// first block) the B blocks' sums it receives -- unless those would leave room
+// for three blocks on an SM instead of four (windows of 15 samples and more,
+// BF16 storage from 13): the first block then reads them where they are, and
+// the others wait for it (w = 8, 258 units x 1008 traces: 93 us, against 105 us
+// at three blocks an SM and 99 us through global scratch).
+template <typename T>
+constexpr bool split_pulls(int W) {
+  return split_set_bytes<T>(W) * size_t(kSplitWarps + kSplitSmallBlocks) > 55 * 1024;
+}
+template <typename T>
+constexpr size_t split_smem_bytes_of(int B, int W) {
+  return split_set_bytes<T>(W) * size_t(kSplitWarps + (B > 1 && !split_pulls<T>(W) ? B : 0));
+}
 inline size_t split_smem_bytes(int B, int W, bool bf16) {
-  const size_t set = bf16 ? split_set_bytes<__nv_bfloat16>(W) : split_set_bytes<float>(W);
-  return set * size_t(kSplitWarps + (B > 1 ? B : 0));
+  return bf16 ? split_smem_bytes_of<__nv_bfloat16>(B, W) : split_smem_bytes_of<float>(B, W);
 }
 // k_semblance_short and k_search_short: the unit's B sums
 inline size_t short_smem_bytes(int B, int W, bool bf16) {
@@ -510,15 +521,17 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 4) k_semblance_split(const E
   namespace cg = cooperative_groups;
   const cg::cluster_group cl = cg::this_cluster();
   extern __shared__ __align__(16) unsigned char split_smem[];
+  constexpr bool PULL = split_pulls<T>(W);
   const int B = a.split_blocks;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const long long unit = blockIdx.x / B;
   const int rank = int(blockIdx.x - unit * B);
   double* part_Ed = reinterpret_cast<double*>(split_smem);  // [S][64], then [B][64]
   double* recv_Ed = part_Ed + S * 64;
-  float* part = reinterpret_cast<float*>(part_Ed + (Chunk<T>::kF64 ? (S + (B > 1 ? B : 0)) * 64 : 0));
+  const int sets = S + (B > 1 && !PULL ? B : 0);
+  float* part = reinterpret_cast<float*>(part_Ed + (Chunk<T>::kF64 ? sets * 64 : 0));
   float* recv = part + S * R * 64;  // [B][R][64], in the cluster's first block
-  if (B > 1) cluster_arrive_relaxed();  // met by cluster_wait below: every block has started
+  if (B > 1 && !PULL) cluster_arrive_relaxed();  // met by cluster_wait below: every block has started
   const long long q0 = unit * 64 + lane, q1 = q0 + 32;
   Lane L0, L1;
   const bool v0 = lane_setup<OP, true>(a, q0, L0);
@@ -568,7 +581,7 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 4) k_semblance_split(const E
   // the block's sums, slices in order: to the cluster's first block
   float* to = part;
   double* to_d = part_Ed;
-  if (B > 1) {
+  if (B > 1 && !PULL) {
     cluster_wait();
     to = cl.map_shared_rank(recv, 0) + rank * R * 64;
     to_d = cl.map_shared_rank(recv_Ed, 0) + rank * 64;
@@ -584,7 +597,8 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 4) k_semblance_split(const E
     for (int v = 0; v < S; ++v) t += part_Ed[v * 64 + threadIdx.x];
     to_d[threadIdx.x] = t;
   }
-  if (B > 1) {
+  double Ed = 0.0;
+  if (B > 1 && !PULL) {
     __syncwarp();
     cluster_arrive();
     if (rank) return;  // done with: nothing of this block's shared memory is read by others
@@ -594,16 +608,25 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 4) k_semblance_split(const E
       for (int b = 0; b < B; ++b) t = __fadd_rn(t, recv[b * R * 64 + i]);
       part[i] = t;
     }
+    if (Chunk<T>::kF64 && threadIdx.x < 64)
+      for (int b = 0; b < B; ++b) Ed += recv_Ed[b * 64 + threadIdx.x];
+  } else if (B > 1) {
+    cl.sync();
+    if (rank == 0) {
+      for (int i = threadIdx.x; i < R * 64; i += NT) {
+        float t = 0.f;
+        for (int b = 0; b < B; ++b) t = __fadd_rn(t, cl.map_shared_rank(part, b)[i]);
+        part[i] = t;
+      }
+      if (Chunk<T>::kF64 && threadIdx.x < 64)
+        for (int b = 0; b < B; ++b) Ed += cl.map_shared_rank(part_Ed, b)[threadIdx.x];
+    }
+    cl.sync();  // no block leaves while its sums are read
+    if (rank) return;
   }
   __syncthreads();
   if (threadIdx.x < 64) {
-    double Ed = 0.0;
-    if (Chunk<T>::kF64) {
-      if (B > 1)
-        for (int b = 0; b < B; ++b) Ed += recv_Ed[b * 64 + threadIdx.x];
-      else
-        Ed = part_Ed[threadIdx.x];
-    }
+    if (Chunk<T>::kF64 && B == 1) Ed = part_Ed[threadIdx.x];
     finish_pair<W, T>(a, unit * 64 + threadIdx.x, size[threadIdx.x], part + threadIdx.x, Ed);
   }
 }
