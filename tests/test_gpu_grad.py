@@ -134,3 +134,35 @@ def test_cmp_gradient_and_polish():
                                           th.cpu().numpy()[:, None, :])[:, 0]
     assert np.max(np.abs(ref - Sp)) <= 1e-5
     ctx.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+def test_autograd_keeps_the_adjoint_of_its_forward(storage):
+    """One adjoint launch serves the forward and every backward of a call;
+    without a gradient to follow the call is tt_semblance_eval; a theta
+    changed in place before the backward is refused."""
+    wl = configs.cmp_search(3, ns=60)
+    ctx = tt.tt_ctx_create(wl.traces, wl.mid, wl.off, wl.problem, None, storage=storage,
+                           device=dev())
+    rng = np.random.default_rng(4)
+    theta = to_dev(wl.de.lo[0] + rng.uniform(0, 1, (60, 2, 1)) * (wl.de.hi[0] - wl.de.lo[0]))
+    S, G = tt.tt_semblance_grad(ctx, theta)
+    E = tt.tt_semblance_eval(ctx, theta)
+    th = theta.clone().requires_grad_(True)
+    tt.tt_ctx_stats(ctx, reset=True)
+    out = tt.semblance(ctx, th)
+    out.sum().backward(retain_graph=True)
+    assert torch.equal(th.grad, G)
+    (2 * out).sum().backward()
+    assert torch.equal(th.grad, G + 2 * G)
+    assert tt.tt_ctx_stats(ctx)["launches"] == (1 if storage == "f32" else 2)
+    assert torch.equal(out, S if storage == "f32" else E)
+    with torch.no_grad():
+        assert torch.equal(tt.semblance(ctx, th), E)
+    assert torch.equal(tt.semblance(ctx, theta), E) and not tt.semblance(ctx, theta).requires_grad
+    out = tt.semblance(ctx, th)
+    with torch.no_grad():
+        th.mul_(1.0)
+    with pytest.raises(RuntimeError, match="inplace"):
+        out.sum().backward()
+    ctx.close()
