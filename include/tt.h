@@ -23,7 +23,9 @@
  *    asynchronous launch. tt_last_error() gives a message.
  *  - A context may be used from one host thread at a time; calls on
  *    different streams that share a context's scratch (tt_search,
- *    tt_ens_search, tt_neighbor_exchange, tt_polish) must not overlap.
+ *    tt_search_slab, tt_ens_search, tt_neighbor_exchange, tt_polish, and
+ *    evaluations under TT_KERNEL_PERSISTENT, which share one work counter)
+ *    must not overlap.
  *
  * Notation (the paper's): a domain is one zero-offset sample (m0, it0),
  * t0 = it0 dt (Sec. 2.1, "index-vector point (t, tr)"); its aperture is the

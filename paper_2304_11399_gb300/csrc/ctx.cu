@@ -612,7 +612,7 @@ extern "C" tt_status tt_ctx_create(tt_ctx** out, const tt_gathers* ga, const tt_
       TRY(dalloc(&c->jade_CR, nd * np), "alloc adaptation");
     }
   }
-  TRY(dalloc(&c->queue, 1), "alloc queue");
+  TRY(dalloc(&c->queue, 2), "alloc queue");
   TRY(dalloc(&c->probe, tt::kProbeFloats), "alloc probe window");
   {
     size_t nd = size_t(c->n_dom), Dz = size_t(D);

@@ -216,8 +216,10 @@ tt_status ens_body(tt_ctx* c, const tt_ens_cfg& e, float* bth, float* bS, cudaSt
   // The interpolated samples of a step (interpolate, evaluate, keep) only
   // touch that trace's skipped samples, which the next steps of the stage do
   // not read; they run on the side stream, overlapping the next step, with
-  // their maps and buffers double-buffered by step parity. A step waits for the side work of the step two before it
-  // (which used the same buffers); every stage ends with a join.
+  // their maps and buffers double-buffered by step parity and a work counter of
+  // their own (a persistent launch clears its counter and takes units from it).
+  // A step waits for the side work of the step two before it (which used the
+  // same buffers); every stage ends with a join.
   if (!c->side_stream) {
     cudaError_t r = cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking);
     for (int k = 0; r == cudaSuccess && k < 4; ++k)
@@ -332,6 +334,7 @@ tt_status ens_body(tt_ctx* c, const tt_ens_cfg& e, float* bth, float* bS, cudaSt
         tt::EvalArgs ei = c->eval_args(th_skp, 1, S_skp);
         ei.n_dom = n_skp_loc;
         ei.dom_map = map_skp;
+        ei.queue = c->queue + 1;
         STEP(c->semblance(ei, s2, false), "ens evaluate interpolated");
         calls += (unsigned long long)active * g.n_skp;
         k_ens_keep<<<blocks(n_skp_loc), 256, 0, s2>>>(n_skp_loc, D, map_skp, th_skp, S_skp, bth,

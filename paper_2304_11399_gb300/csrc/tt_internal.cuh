@@ -222,7 +222,9 @@ struct tt_ctx {
   float *pol_th = nullptr, *pol_g = nullptr, *pol_S = nullptr, *pol_bth = nullptr,
         *pol_bS = nullptr;
   int* d_err = nullptr;     // device-side validation flag
-  unsigned long long* queue = nullptr;  // persistent-kernel work counter
+  // persistent-kernel work counters: one of the calls, one of the launches that
+  // the ENS sweep runs beside them on its side stream (each launch clears its own)
+  unsigned long long* queue = nullptr;
   float* probe = nullptr;   // window and sink of the L1 probe (kProbeFloats)
   // a side stream: the ENS sweep evaluates each step's interpolated samples
   // concurrently with the next step

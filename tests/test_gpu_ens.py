@@ -169,3 +169,22 @@ def test_full_line_sweep_in_the_bench_configuration():
     ref = oracle.semblance.semblance_many(wl.traces, wl.mid, wl.off, prob, th[doms][:, None, :],
                                           domains=doms)[:, 0]
     assert np.max(np.abs(ref - S[doms])) <= 1e-5
+
+
+def test_persistent_evaluations_on_both_streams():
+    """Unsplit persistent launches of more units than warps fit the GPU, on the
+    main stream and beside them on the side stream: each takes its units from a
+    counter of its own, so the sweep gives the bits of the grid-mapped form. (A
+    shared counter, cleared by one launch while the other counts, leaves units
+    out.) 100 buckets of two traces x 480 estimated samples x 16 members are
+    12,000 units, the 960 samples interpolated beside them 1,500."""
+    wl = configs.crs_line(5, n_cmp=200, ns=1440, n_events=4, ap_half=1, np_=16, tau_max=0.7)
+    ctx = tt.tt_ctx_create(wl.traces, wl.mid, wl.off, wl.problem, wl.de, device=dev())
+    tt.tt_ctx_set_option(ctx, "split", False)
+    outs = []
+    for kernel in ("packed", "persistent"):
+        tt.tt_ctx_set_option(ctx, "kernel", kernel)
+        outs.append(tt.tt_ens_search(ctx, 16, 1, 16, 1, 2, 1, 2))
+    ctx.close()
+    assert outs[0][2] == outs[1][2]
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
