@@ -432,8 +432,8 @@ extern "C" tt_status tt_ctx_create(tt_ctx** out, const tt_gathers* ga, const tt_
     return tt_fail(nullptr, TT_ERR_UNSUPPORTED, "padded trace buffer exceeds 2^32 samples");
   const int D = tt::op_dim(pr->op);
   if (cfg) {
-    if (cfg->np < 4 || cfg->np > 1024)
-      return tt_fail(nullptr, TT_ERR_INVALID_ARG, "np %d outside 4..1024", cfg->np);
+    if (cfg->np < 4 || cfg->np > tt::kMaxNP)
+      return tt_fail(nullptr, TT_ERR_INVALID_ARG, "np %d outside 4..%d", cfg->np, tt::kMaxNP);
     if (cfg->ng < 0) return tt_fail(nullptr, TT_ERR_INVALID_ARG, "ng < 0");
     if (!(cfg->F >= 0.f && cfg->F <= 2.f) || !(cfg->CR >= 0.f && cfg->CR <= 1.f))
       return tt_fail(nullptr, TT_ERR_INVALID_ARG, "F must be in [0,2], CR in [0,1]");

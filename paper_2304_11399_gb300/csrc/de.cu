@@ -140,8 +140,10 @@ cudaError_t launch_de_step(const DeArgs& a, cudaStream_t s) {
   if (a.n_dom == 0) return cudaSuccess;
   void (*fn)(const DeArgs) = a.D == 1 ? k_de_step<1> : a.D == 3 ? k_de_step<3> : k_de_step<5>;
   const size_t sm = a.gen == 0 ? 0 : size_t(kWarps) * a.NP * (a.D + 1) * sizeof(float);
-  if (sm > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+  if (sm > 48 * 1024) {  // the kernel's limit, shared by every context: always the same figure
+    const size_t most = size_t(kWarps) * kMaxNP * (a.D + 1) * sizeof(float);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         int(most));
     if (e != cudaSuccess) return e;
   }
   fn<<<(a.n_dom + kWarps - 1) / kWarps, kWarps * 32, sm, s>>>(a);

@@ -35,11 +35,13 @@ KFn pick(int kind, const EvalArgs& a, bool mv) {
 }
 
 // A block's shared memory above 48 KB, the kernel's own arrays included, has
-// to be asked for.
+// to be asked for. The limit belongs to the kernel, for every context and host
+// thread: `most` is the largest size any launch of fn takes, so that no call
+// lowers the limit between another's setting it and launching.
 template <typename Fn>
-cudaError_t allow_smem(Fn fn, size_t bytes) {
-  if (bytes <= 40 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+cudaError_t allow_smem(Fn fn, size_t most) {
+  if (most <= 40 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(most));
 }
 
 // Sums of eight slices per pair of a split launch (see semblance_kernels.cuh).
@@ -70,7 +72,7 @@ cudaError_t launch_split(EvalArgs& a, long long units, bool mv, cudaStream_t s) 
   const KFn fn = pick(sk::kKindSplit, a, mv);
   if (!fn) return cudaErrorInvalidValue;
   const size_t smem = sk::split_smem_bytes(B, a.W, bf);
-  cudaError_t e = allow_smem(fn, smem);
+  cudaError_t e = allow_smem(fn, sk::split_smem_bytes(kSplitTinyBlocks, a.W, bf));
   if (e == cudaSuccess && B > 8)  // more blocks than every device has to offer
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
@@ -241,8 +243,9 @@ cudaError_t launch_fused_search(const EvalArgs& a, const DeArgs& de, const Fused
   if (!fn || a.P > 64) return cudaErrorInvalidValue;
   const int B = split_blocks(((long long)a.n_dom * a.P + 63) / 64, a.n_sm);
   const int per = 64 / a.P;
-  const size_t smem = sk::short_smem_bytes(B, a.W, a.storage == TT_STORE_BF16);
-  const cudaError_t e = allow_smem(fn, smem);
+  const bool bf = a.storage == TT_STORE_BF16;
+  const size_t smem = sk::short_smem_bytes(B, a.W, bf);
+  const cudaError_t e = allow_smem(fn, sk::short_smem_bytes(kSplitTinyBlocks, a.W, bf));
   if (e != cudaSuccess) return e;
   fn<<<(a.n_dom + per - 1) / per, 32 * B, smem, s>>>(a, de, f);
   return cudaGetLastError();

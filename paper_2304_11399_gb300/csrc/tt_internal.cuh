@@ -34,6 +34,7 @@ constexpr int kPadFront = 8;
 constexpr int kPadBack = 24;
 constexpr int kBlock = 256;
 constexpr int kProbeFloats = 8192 + 1;
+constexpr int kMaxNP = 1024;     // largest population of a search
 constexpr int kOrderMaxP = 256;  // largest population the member order handles
 // automatic member order: on when the mean aperture holds at least this many traces
 constexpr double kOrderMinMeanAperture = 768.0;

@@ -1,5 +1,7 @@
 """Forms of a launch that compute the same thing, compared at the sizes where
 the forms change or a tile is ragged."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -155,3 +157,42 @@ def test_fused_search_equals_stepwise(n_dom, np_, ng, op, w, storage, ns, sizes,
     assert few["launches"] < many["launches"] or ng == 0
     assert few["trace_evals"] == many["trace_evals"]
     assert few["semblance_launches"] == many["semblance_launches"]
+
+
+@pytest.mark.parametrize("storage,w", [("f32", 5), ("f32", 6), ("bf16", 5)])
+def test_two_contexts_on_two_threads(storage, w):
+    """Launches of the same kernels with different amounts of shared memory, a
+    context and a stream per host thread: evaluations of 8 and of 80 units
+    (clusters of 9 and of 7 blocks) and searches of them (9 and 7 warps). A limit
+    that one thread lowers would refuse the other's launch."""
+    x, mid, off = _line(60, 300)
+    errors, start = [], threading.Barrier(2, timeout=60)
+
+    def run(n_dom):
+        try:
+            s = torch.cuda.Stream(device=dev())
+            with torch.cuda.stream(s):
+                prob = _problem(n_dom, (100,), 60, 300, w=w)
+                ctx = tt.tt_ctx_create(x, mid, off, prob, _cfg(1, 64, 2), storage=storage,
+                                       device=dev())
+                tt.tt_ctx_set_option(ctx, "search_graph", False)
+                th = to_dev(random_theta(n_dom, 64, *BOUNDS[1], 7))
+                S = tt.tt_semblance_eval(ctx, th)
+                best = tt.tt_search(ctx)[1]
+                start.wait()
+                for _ in range(500):
+                    S1 = tt.tt_semblance_eval(ctx, th)
+                    best1 = tt.tt_search(ctx)[1]
+                assert torch.equal(S, S1) and torch.equal(best, best1)
+                s.synchronize()
+                ctx.close()
+        except BaseException as e:  # reported by the main thread
+            errors.append(e)
+            start.abort()
+
+    threads = [threading.Thread(target=run, args=(n,)) for n in (8, 80)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
