@@ -961,9 +961,16 @@ __global__ void __launch_bounds__(kBlock) k_semblance_scalar(const EvalArgs a) {
 // u = 0 contributes nothing, and positions clamped to the all-zero window give
 // zero by themselves.
 
-// d S / d u of one trace over u: the factor every parameter's chain shares.
-__device__ __forceinline__ float over_u(float dSdu, float u) {
-  return u > 0.f ? __fmul_rn(dSdu, rcp_approx(u)) : 0.f;
+// 1 / u of two positions, 0 where u = 0 (a product rather than a skipped term, so
+// that a NaN passes on as it does in the unsplit form). The hardware's reciprocal
+// is up to 1 ulp off; a Newton step y + y (1 - u y) on the FMA pipe leaves the
+// rounding of the result, as the unsplit form's division has. Positions are below
+// 2^25 and, where not 0, above 1e-19: nothing here leaves the normal range.
+__device__ __forceinline__ float2 inv_u(float u0, float u1) {
+  const float2 u = make_float2(u0, u1);
+  const float2 y = make_float2(u0 > 0.f ? rcp_approx(u0) : 0.f, u1 > 0.f ? rcp_approx(u1) : 0.f);
+  const float2 e = __ffma2_rn(__fmul2_rn(u, make_float2(-1.f, -1.f)), y, make_float2(1.f, 1.f));
+  return __ffma2_rn(y, e, y);
 }
 
 // Pass 2 of one pair over aperture entries [r0, r1): G += the entries' terms
@@ -988,7 +995,7 @@ __device__ __forceinline__ void adj_scalar(const EvalArgs& a, const Lane& L, int
       sg = fmaf(s[k], gk, sg);
       ag = fmaf(ak, gk, ag);
     }
-    const float c = over_u(fmaf(alpha, sg, __fmul_rn(nbeta, ag)), P.u);
+    const float c = __fmul_rn(fmaf(alpha, sg, __fmul_rn(nbeta, ag)), inv_u(P.u, P.u).x);
     const float hc = __fmul_rn(0.5f, c), cq = __fmul_rn(c, P.q);
     if (OP == TT_OP_FOCRS) {  // dU = 2q dm, 2q dh, dm^2, dm dh, dh^2
       const float hm = __fmul_rn(hc, t4.x), hh = __fmul_rn(hc, t4.y);
@@ -1034,7 +1041,7 @@ __device__ __forceinline__ void adj_packed(const EvalArgs& a, const Lane& L0, co
       ag = __ffma2_rn(ak, gk, ag);
     }
     const float2 d = __ffma2_rn(alpha, sg, __fmul2_rn(nbeta, ag));
-    const float2 c = make_float2(over_u(d.x, P0.u), over_u(d.y, P1.u));
+    const float2 c = __fmul2_rn(d, inv_u(P0.u, P1.u));
     const float2 hc = __fmul2_rn(half, c), cq = __fmul2_rn(c, make_float2(P0.q, P1.q));
     const float2 tx = make_float2(t4.x, t4.x), ty = make_float2(t4.y, t4.y),
                  tz = make_float2(t4.z, t4.z);
@@ -1055,28 +1062,29 @@ __device__ __forceinline__ void adj_packed(const EvalArgs& a, const Lane& L0, co
   }
 }
 
-// S, alpha and -beta from a pair's sums (all zero when the energy is 0).
+// S, alpha and -beta from a pair's sums; false (and both zero) when the energy
+// is 0 or NaN. An infinite energy has a gradient like its S: NaN.
 template <typename T>
-__device__ __forceinline__ float grad_factors(float Q, int N, float E, double Ed, float& alpha,
-                                              float& nbeta) {
-  const float S = normalise<T>(Q, N, E, Ed);
+__device__ __forceinline__ bool grad_factors(float Q, int N, float E, double Ed, float& S,
+                                             float& alpha, float& nbeta) {
+  S = normalise<T>(Q, N, E, Ed);
   const float En = Chunk<T>::kF64 ? float(Ed) : E;
   const bool ok = En > 0.f;
   alpha = ok ? 2.f / (float(N) * En) : 0.f;
   nbeta = ok ? -2.f * S / En : 0.f;
-  return S;
+  return ok;
 }
 
-// dS of pair q: the 1/dt factors; zero when the energy is 0 (alpha = 0).
+// dS of pair q: the 1/dt factors; zero without an energy to divide by.
 template <int OP>
-__device__ __forceinline__ void store_grad(const EvalArgs& a, long long q, float inv_dt,
-                                           float alpha, const float* G) {
+__device__ __forceinline__ void store_grad(const EvalArgs& a, long long q, float inv_dt, bool ok,
+                                           const float* G) {
   constexpr int D = op_dim(OP);
   constexpr int n1 = OP == TT_OP_FOCRS ? 2 : OP == TT_OP_CRS ? 1 : 0;  // slopes: 1/dt
   const float i2 = inv_dt * inv_dt;
   float* out = a.dS + q * D;
 #pragma unroll
-  for (int d = 0; d < D; ++d) out[d] = alpha > 0.f ? G[d] * (d < n1 ? inv_dt : i2) : 0.f;
+  for (int d = 0; d < D; ++d) out[d] = ok ? G[d] * (d < n1 ? inv_dt : i2) : 0.f;
 }
 
 // K2 with one pair per thread, both passes in entry order: the form of the
@@ -1286,15 +1294,16 @@ __global__ void __launch_bounds__(32 * kGradWarps, 3) k_semblance_grad_split(con
     tot[i] = t;
   }
   __syncthreads();
+  bool ok = false;  // thread p < 64: pair p has an energy
   if (threadIdx.x < 64 && size[threadIdx.x] >= 0) {
     const int p = threadIdx.x;
-    float Q = 0.f, al, nb;
+    float Q = 0.f, Sv, al, nb;
 #pragma unroll
     for (int k = 0; k < K; ++k) Q = fmaf(tot[k * 64 + p], tot[k * 64 + p], Q);
     double Ed = 0.0;
     if (Chunk<T>::kF64)
       for (int b = 0; b < B; ++b) Ed += B > 1 ? cl.map_shared_rank(blk_Ed, b)[p] : blk_Ed[p];
-    const float Sv = grad_factors<T>(Q, size[p], tot[K * 64 + p], Ed, al, nb);
+    ok = grad_factors<T>(Q, size[p], tot[K * 64 + p], Ed, Sv, al, nb);
     fac[p] = al;
     fac[64 + p] = nb;
     if (rank == 0) a.S[unit * 64 + p] = Sv;
@@ -1350,7 +1359,7 @@ __global__ void __launch_bounds__(32 * kGradWarps, 3) k_semblance_grad_split(con
         for (int b = 0; b < B; ++b)
           G[d] = __fadd_rn(G[d], B > 1 ? cl.map_shared_rank(blk, b)[d * 64 + p] : blk[d * 64 + p]);
       }
-      store_grad<OP>(a, unit * 64 + p, L.inv_dt, fac[p], G);
+      store_grad<OP>(a, unit * 64 + p, L.inv_dt, ok, G);
     }
   }
   if (B > 1) cl.sync();  // no block leaves while another may read its sums

@@ -196,3 +196,36 @@ def test_two_contexts_on_two_threads(storage, w):
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+@pytest.mark.parametrize("n_dom,P,sizes,op,w,ns", [
+    (300, 1, (200,), 0, 5, 300), (300, 1, (300,), 1, 3, 300), (9000, 1, (300,), 2, 5, 2200)])
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+@pytest.mark.parametrize("bad", [float("inf"), 1e25, float("nan")])
+def test_gradient_of_infinite_energy(n_dom, P, sizes, op, w, ns, storage, bad):
+    """Windows with an infinite energy (an infinite sample, or 1e25, whose square
+    is) have S = dS = NaN in the split gradient as in the unsplit one; with a NaN
+    energy both are 0. BF16 storage sums the split form's energy in FP64, where
+    1e25 squared is finite: not compared."""
+    if storage == "bf16" and bad == 1e25:
+        pytest.skip("finite in the split form's FP64 energy")
+    x, mid, off = _line(60, ns)
+    off[7] = 5.0  # an early window of every aperture that holds trace 7
+    x[7, 40:60] = bad
+    prob = _problem(n_dom, sizes, 60, ns, op, w)
+    bounds = BOUNDS[op] if op else ((1 / 4500 ** 2,), (1 / 1400 ** 2,))
+    th = to_dev(random_theta(n_dom, P, *bounds, 5))
+    ctx = tt.tt_ctx_create(x, mid, off, prob, None, storage=storage, device=dev())
+    out = []
+    for split in (True, False):
+        tt.tt_ctx_set_option(ctx, "split", split)
+        out.append(tt.tt_semblance_grad(ctx, th))
+        assert torch.equal(out[-1][0].isnan(), tt.tt_semblance_eval(ctx, th).isnan())
+    ctx.close()
+    (S, G), (S0, G0) = out
+    assert torch.equal(S.isnan(), S0.isnan()) and torch.equal(G.isnan(), G0.isnan())
+    assert torch.equal(S == 0, S0 == 0) and torch.equal((G == 0).all(-1), (G0 == 0).all(-1))
+    if bad == bad:
+        assert S.isnan().any() and G[S.isnan()].isnan().all()
+    else:
+        assert (S == 0).any() and not S.isnan().any() and not G.isnan().any()
