@@ -106,6 +106,11 @@ bool grad_split(const EvalArgs& a, long long units) {
          (a.mean_ap >= 256.f || (a.mean_ap >= 16.f && units < 16ll * a.n_sm));
 }
 
+// Pairs times aperture entries up to which a differentiated evaluation takes the
+// adjoint at once: there it runs 20 to 45 us, the evaluation 20, and a call takes
+// 33 us to issue (4 million: 52 to 59 us).
+constexpr double kGradTogetherMax = 2097152.0;
+
 // The cluster has the forward launch's B blocks (1008 traces, clusters of 1 / 2
 // / 4 / 8: 24 units 115 / 66 / 38 / 28 us, 282 units 308 / 235 / 207 / 217 us,
 // 938 units 647 / 562 / 577 / 680 us, at two blocks per SM: the rule's 9, 7 and
@@ -145,7 +150,7 @@ cudaError_t launch(const EvalArgs& a, cudaStream_t s, bool grad) {
   EvalArgs b = a;
   if (grad) {
     const long long units = (n + 63) / 64;
-      if (grad_split(a, units)) return launch_grad_split(a, units, mv, s);
+    if (a.sums || grad_split(a, units)) return launch_grad_split(a, units, mv, s);
     // few pairs: several entries in flight, in small blocks that spread over the SMs
     const bool few = n < 768ll * a.n_sm;
     fn = pick(few ? sk::kKindGradAhead : sk::kKindGrad, a, mv);
@@ -216,6 +221,30 @@ cudaError_t launch_stack(const EvalArgs& a, float* out, cudaStream_t s) {
 }
 
 cudaError_t launch_semblance_grad(const EvalArgs& a, cudaStream_t s) { return launch(a, s, true); }
+
+// How a differentiated evaluation runs: its value now, its gradient later or
+// never. The sums of a split evaluation are kept and the gradient starts from
+// them (60,000 domains x 1008 traces: the value 197 us, with its gradient 483 us
+// through autograd, against 459 and 478 us with the adjoint at once and 197 and
+// 675 us with a launch of each; 300,000 x 144: 129 and 336 us, 307 and 325 us, 129
+// and 460 us). Where both passes are no longer than a call takes to issue, the
+// adjoint gives value and gradient at once (2,000 x 1008: 34 and 221 us against 38
+// and 301 us, which is host time). What the evaluation does not split, or holds
+// apertures too short for split gradients, is evaluated and differentiated by
+// launches of their own.
+int grad_plan(const EvalArgs& a) {
+  const long long n = (long long)a.n_dom * a.P, units = (n + 63) / 64;
+  if (!a.split || n == 0 || units >= (long long)a.n_sm * kSplitUnitsPerSm || a.mean_ap < 16.f)
+    return TT_GRAD_SEPARATE;
+  return double(n) * a.mean_ap <= kGradTogetherMax && grad_split(a, units) ? TT_GRAD_TOGETHER
+                                                                           : TT_GRAD_SUMS;
+}
+
+size_t grad_sums_bytes(const EvalArgs& a) {
+  const size_t units = ((size_t)a.n_dom * a.P + 63) / 64;
+  return a.storage == TT_STORE_BF16 ? units * sk::split_set_bytes<__nv_bfloat16>(a.W)
+                                    : units * sk::split_set_bytes<float>(a.W);
+}
 
 // Apertures of up to 160 traces, or of 1.5 per unit where the 64 slots of a
 // block are nearly full: DE 32 x 30 on 38 / 150 / 300 units of 48 traces 144 /
@@ -336,6 +365,55 @@ extern "C" tt_status tt_semblance_grad(tt_ctx* ctx, const float* theta, int32_t 
     return tt_fail(ctx, TT_ERR_INVALID_ARG, "NULL array");
   tt::EvalArgs a = ctx->eval_args(theta, P, S);
   a.dS = dS;
+  return tt_cuda_check(ctx, ctx->semblance(a, static_cast<cudaStream_t>(stream), true),
+                       "semblance gradient launch");
+}
+
+extern "C" tt_status tt_semblance_grad_plan(tt_ctx* ctx, int32_t P, int32_t* plan,
+                                            uint64_t* bytes) {
+  if (!ctx) return tt_fail(nullptr, TT_ERR_INVALID_ARG, "ctx is NULL");
+  if (P < 1) return tt_fail(ctx, TT_ERR_INVALID_ARG, "P must be >= 1");
+  if (!plan || !bytes) return tt_fail(ctx, TT_ERR_INVALID_ARG, "plan or bytes is NULL");
+  const tt::EvalArgs a = ctx->eval_args(nullptr, P, nullptr);
+  *plan = tt::grad_plan(a);
+  *bytes = *plan == TT_GRAD_SUMS ? tt::grad_sums_bytes(a) : 0;
+  return TT_OK;
+}
+
+namespace {
+
+// The two parts of a buffer of sums (the same whatever the launch's slices).
+void set_sums(tt::EvalArgs& a, void* sums) {
+  const size_t units = ((size_t)a.n_dom * a.P + 63) / 64;
+  a.sums_Ed = a.storage == TT_STORE_BF16 ? static_cast<double*>(sums) : nullptr;
+  a.sums = a.sums_Ed ? reinterpret_cast<float*>(a.sums_Ed + units * 64)
+                     : static_cast<float*>(sums);
+}
+
+}  // namespace
+
+extern "C" tt_status tt_semblance_eval_sums(tt_ctx* ctx, const float* theta, int32_t P, float* S,
+                                            void* sums, void* stream) {
+  if (!ctx) return tt_fail(nullptr, TT_ERR_INVALID_ARG, "ctx is NULL");
+  if (P < 1) return tt_fail(ctx, TT_ERR_INVALID_ARG, "P must be >= 1");
+  if (!theta || !S || !sums) return tt_fail(ctx, TT_ERR_INVALID_ARG, "NULL array");
+  tt::EvalArgs a = ctx->eval_args(theta, P, S);
+  if (tt::grad_plan(a) != TT_GRAD_SUMS)
+    return tt_fail(ctx, TT_ERR_INVALID_ARG, "this launch keeps no sums");
+  set_sums(a, sums);
+  return tt_cuda_check(ctx, ctx->semblance(a, static_cast<cudaStream_t>(stream), false),
+                       "semblance launch");
+}
+
+extern "C" tt_status tt_semblance_grad_sums(tt_ctx* ctx, const float* theta, int32_t P,
+                                            const void* sums, float* dS, void* stream) {
+  if (!ctx) return tt_fail(nullptr, TT_ERR_INVALID_ARG, "ctx is NULL");
+  if (P < 1) return tt_fail(ctx, TT_ERR_INVALID_ARG, "P must be >= 1");
+  if (ctx->n_dom > 0 && (!theta || !sums || !dS))
+    return tt_fail(ctx, TT_ERR_INVALID_ARG, "NULL array");
+  tt::EvalArgs a = ctx->eval_args(theta, P, nullptr);
+  a.dS = dS;
+  set_sums(a, const_cast<void*>(sums));
   return tt_cuda_check(ctx, ctx->semblance(a, static_cast<cudaStream_t>(stream), true),
                        "semblance gradient launch");
 }

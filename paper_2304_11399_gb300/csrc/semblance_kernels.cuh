@@ -503,11 +503,18 @@ inline size_t short_smem_bytes(int B, int W, bool bf16) {
 }
 
 // S of pair q (row entry p) from its summed rows; N = -1 marks an absent pair.
+// The rows themselves are kept where a gradient is to follow (a.sums).
 template <int W, typename T>
 __device__ __forceinline__ void finish_pair(const EvalArgs& a, long long q, int N,
                                             const float* tot, double Ed) {
   constexpr int K = 2 * W + 1;
   if (N < 0) return;
+  if (a.sums) {
+    float* out = a.sums + (q >> 6) * ((K + 1) * 64) + (q & 63);
+#pragma unroll
+    for (int k = 0; k <= K; ++k) out[k * 64] = tot[k * 64];
+    if (Chunk<T>::kF64) a.sums_Ed[q] = Ed;
+  }
   float Q = 0.f;
 #pragma unroll
   for (int k = 0; k < K; ++k) Q = fmaf(tot[k * 64], tot[k * 64], Q);
@@ -1232,65 +1239,69 @@ __global__ void __launch_bounds__(32 * kGradWarps, 3) k_semblance_grad_split(con
   const bool both = v0 && v1 && same_aperture(L0, L1);
   __shared__ int size[64];
   if (w == 0) keep_sizes(size, lane, v0, L0, v1, L1);
-  // pass 1
   int r0 = 0, r1 = 0;
-  if (both) {
-    slice_of(L0, S * B, rank * S + w, r0, r1);
-    float2 s[K];
+  if (both) slice_of(L0, S * B, rank * S + w, r0, r1);
+  if (!a.sums) {  // pass 1, unless the forward launch has kept its sums
+    if (both) {
+      float2 s[K];
 #pragma unroll
-    for (int k = 0; k < K; ++k) s[k] = make_float2(0.f, 0.f);
-    float2 E = make_float2(0.f, 0.f);
-    double Ed0 = 0.0, Ed1 = 0.0;
-    acc_packed<OP, W, T, MV>(a, L0, L1, r0, r1, s, E, Ed0, Ed1);
+      for (int k = 0; k < K; ++k) s[k] = make_float2(0.f, 0.f);
+      float2 E = make_float2(0.f, 0.f);
+      double Ed0 = 0.0, Ed1 = 0.0;
+      acc_packed<OP, W, T, MV>(a, L0, L1, r0, r1, s, E, Ed0, Ed1);
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-      part[(w * R + k) * 64 + lane] = s[k].x;
-      part[(w * R + k) * 64 + lane + 32] = s[k].y;
-    }
-    part[(w * R + K) * 64 + lane] = E.x;
-    part[(w * R + K) * 64 + lane + 32] = E.y;
-    if (Chunk<T>::kF64) {
-      part_Ed[w * 64 + lane] = Ed0;
-      part_Ed[w * 64 + lane + 32] = Ed1;
-    }
-  } else {
-    for (int h = 0; h < 2; ++h) {
-      float s[K], E = 0.f;
-      double Ed = 0.0;
-#pragma unroll
-      for (int k = 0; k < K; ++k) s[k] = 0.f;
-      if (h ? v1 : v0) {
-        const Lane& L = h ? L1 : L0;
-        slice_of(L, S * B, rank * S + w, r0, r1);
-        acc_scalar<OP, W, T, MV>(a, L, r0, r1, s, E, Ed);
+      for (int k = 0; k < K; ++k) {
+        part[(w * R + k) * 64 + lane] = s[k].x;
+        part[(w * R + k) * 64 + lane + 32] = s[k].y;
       }
-      const int p = lane + 32 * h;
+      part[(w * R + K) * 64 + lane] = E.x;
+      part[(w * R + K) * 64 + lane + 32] = E.y;
+      if (Chunk<T>::kF64) {
+        part_Ed[w * 64 + lane] = Ed0;
+        part_Ed[w * 64 + lane + 32] = Ed1;
+      }
+    } else {
+      for (int h = 0; h < 2; ++h) {
+        float s[K], E = 0.f;
+        double Ed = 0.0;
 #pragma unroll
-      for (int k = 0; k < K; ++k) part[(w * R + k) * 64 + p] = s[k];
-      part[(w * R + K) * 64 + p] = E;
-      if (Chunk<T>::kF64) part_Ed[w * 64 + p] = Ed;
+        for (int k = 0; k < K; ++k) s[k] = 0.f;
+        if (h ? v1 : v0) {
+          const Lane& L = h ? L1 : L0;
+          slice_of(L, S * B, rank * S + w, r0, r1);
+          acc_scalar<OP, W, T, MV>(a, L, r0, r1, s, E, Ed);
+        }
+        const int p = lane + 32 * h;
+#pragma unroll
+        for (int k = 0; k < K; ++k) part[(w * R + k) * 64 + p] = s[k];
+        part[(w * R + K) * 64 + p] = E;
+        if (Chunk<T>::kF64) part_Ed[w * 64 + p] = Ed;
+      }
     }
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < R * 64; i += NT) {
-    float t = 0.f;
+    __syncthreads();
+    for (int i = threadIdx.x; i < R * 64; i += NT) {
+      float t = 0.f;
 #pragma unroll
-    for (int v = 0; v < S; ++v) t = __fadd_rn(t, part[v * R * 64 + i]);
-    blk[i] = t;
+      for (int v = 0; v < S; ++v) t = __fadd_rn(t, part[v * R * 64 + i]);
+      blk[i] = t;
+    }
+    if (Chunk<T>::kF64 && threadIdx.x < 64) {
+      double t = 0.0;
+      for (int v = 0; v < S; ++v) t += part_Ed[v * 64 + threadIdx.x];
+      blk_Ed[threadIdx.x] = t;
+    }
+    if (B > 1) cl.sync(); else __syncthreads();
   }
-  if (Chunk<T>::kF64 && threadIdx.x < 64) {
-    double t = 0.0;
-    for (int v = 0; v < S; ++v) t += part_Ed[v * 64 + threadIdx.x];
-    blk_Ed[threadIdx.x] = t;
-  }
-  if (B > 1) cl.sync(); else __syncthreads();
   // the unit's sums, in every block, over the slice sums that are done with
   float* tot = part;                     // [R][64]
   float* fac = part + R * 64;            // alpha [64], -beta [64]
   float* gsl = fac + 2 * 64;             // [S][D][64]
   for (int i = threadIdx.x; i < R * 64; i += NT) {
     float t = 0.f;
-    for (int b = 0; b < B; ++b) t = __fadd_rn(t, B > 1 ? cl.map_shared_rank(blk, b)[i] : blk[i]);
+    if (a.sums)
+      t = a.sums[unit * (R * 64) + i];
+    else
+      for (int b = 0; b < B; ++b) t = __fadd_rn(t, B > 1 ? cl.map_shared_rank(blk, b)[i] : blk[i]);
     tot[i] = t;
   }
   __syncthreads();
@@ -1301,14 +1312,16 @@ __global__ void __launch_bounds__(32 * kGradWarps, 3) k_semblance_grad_split(con
 #pragma unroll
     for (int k = 0; k < K; ++k) Q = fmaf(tot[k * 64 + p], tot[k * 64 + p], Q);
     double Ed = 0.0;
-    if (Chunk<T>::kF64)
+    if (Chunk<T>::kF64 && a.sums)
+      Ed = a.sums_Ed[unit * 64 + p];
+    else if (Chunk<T>::kF64)
       for (int b = 0; b < B; ++b) Ed += B > 1 ? cl.map_shared_rank(blk_Ed, b)[p] : blk_Ed[p];
     ok = grad_factors<T>(Q, size[p], tot[K * 64 + p], Ed, Sv, al, nb);
     fac[p] = al;
     fac[64 + p] = nb;
-    if (rank == 0) a.S[unit * 64 + p] = Sv;
+    if (rank == 0 && !a.sums) a.S[unit * 64 + p] = Sv;
   }
-  if (B > 1) cl.sync(); else __syncthreads();  // every block has read blk: it is free
+  if (B > 1 && !a.sums) cl.sync(); else __syncthreads();  // every block has read blk: it is free
   // pass 2
   if (both) {
     float2 s[K], G[D];

@@ -63,12 +63,19 @@ struct EvalArgs {
   int split_blocks;         // B of a split launch (set by the launcher)
   int n_sm;                 // SMs of the device (split thresholds, persistent grid)
   unsigned long long* queue;  // persistent mode: work-unit counter, zero at launch
+  // sums of a split launch, 64 pairs at a time: s_k and E [units][2 W + 2][64], BF16
+  // storage's FP64 energies [units * 64]. A forward launch writes them, a
+  // gradient launch starts from them instead of a first pass; NULL: neither.
+  float* sums;
+  double* sums_Ed;
   int n_groups;             // aperture groups of the context
   float mean_ap;            // mean aperture size over the context's domains
 };
 
 cudaError_t launch_semblance(const EvalArgs& a, cudaStream_t s);
 cudaError_t launch_semblance_grad(const EvalArgs& a, cudaStream_t s);
+int grad_plan(const EvalArgs& a);          // TT_GRAD_*
+size_t grad_sums_bytes(const EvalArgs& a); // of a TT_GRAD_SUMS launch
 // Members of each domain of theta (a.theta, a.P <= 256, no domain map) sorted
 // by window position: parameters to theta_out, original slots to slots
 // ([n_dom][P]); evaluate theta_out with slots as the scatter map.

@@ -67,6 +67,7 @@ class Context:
     device: torch.device
     lib: C.CDLL
     storage: str = "f32"
+    loads: int = 0  # reloads of the traces
 
     def close(self):
         if self.handle:
@@ -146,6 +147,7 @@ def tt_ctx_load_traces(ctx: Context, traces, stream=None):
     host = 0 if traces.is_cuda else 1
     st = ctx.lib.tt_ctx_load_traces(ctx.handle, C.c_void_p(traces.data_ptr()), host,
                                     _stream(stream))
+    ctx.loads += 1
     _check(ctx.lib, ctx.handle, st)
 
 
@@ -396,29 +398,76 @@ def tt_ctx_stats(ctx: Context, reset: bool = False) -> dict:
 
 
 class SemblanceFn(torch.autograd.Function):
-    """S(theta) with the hand-written adjoint kernel as its backward. The
-    adjoint needs the sums that make S and returns S as well, so the forward
-    of a differentiated call runs it and keeps dS/dtheta for the backward,
-    which would otherwise walk every aperture a third time (60,000 CRS domains
-    x 1008 traces: 704 -> 505 us a pass, forward and backward). ``adjoint`` says whether a backward can
-    follow (default: whether theta requires a gradient). BF16-stored traces
-    take S from the forward kernel, whose energy is summed in FP64 in every
-    form. theta is saved too: changing it in place before the backward is an
-    error."""
+    """S(theta), as tt_semblance_eval gives it, with the hand-written adjoint
+    kernel as its backward. ``adjoint`` says whether a backward can follow
+    (default: whether theta requires a gradient); without one the call is
+    tt_semblance_eval. With one it runs as tt_semblance_grad_plan says: the
+    evaluation keeps each pair's sums (2w + 2 floats a pair, held until the graph
+    is freed) and the backward is the adjoint's second pass alone; a call of a few
+    microseconds of device time runs the adjoint at once and keeps dS/dtheta; any
+    other is evaluated now and differentiated by the backward. So a value whose
+    backward never comes costs an evaluation (60,000 CRS domains x 1008 traces
+    197 us, with its backward 483 us; as a launch of each, 675 us). The contiguous theta is saved as well: changing it in place before
+    the backward is an error (a copy made of a strided theta is not watched). A
+    backward after tt_ctx_load_traces is taken on the traces then loaded."""
 
     @staticmethod
     def forward(fctx, ctx: Context, theta: torch.Tensor, adjoint=None):
         theta = theta.contiguous()
         if not (fctx.needs_input_grad[1] if adjoint is None else adjoint):
             return tt_semblance_eval(ctx, theta)
-        S, dS = tt_semblance_grad(ctx, theta)
-        fctx.save_for_backward(theta, dS)
-        return S if ctx.storage == "f32" else tt_semblance_eval(ctx, theta)
+        if theta.dim() != 3:
+            raise ValueError("theta must be [n_dom, P, D]")
+        fctx.tt, fctx.loads = ctx, ctx.loads
+        fctx.plan, n_bytes = _grad_plan(ctx, int(theta.shape[1]))
+        if fctx.plan == L.TT_GRAD_SUMS:
+            sums = torch.empty((n_bytes,), dtype=torch.uint8, device=theta.device)
+            fctx.save_for_backward(theta, sums)
+            fctx.stream = torch.cuda.current_stream()  # which autograd's backward runs on too
+            return _eval_sums(ctx, theta, sums, fctx.stream)
+        if fctx.plan == L.TT_GRAD_TOGETHER:
+            S, dS = tt_semblance_grad(ctx, theta)
+            fctx.save_for_backward(theta, dS)
+            return S if ctx.storage == "f32" else tt_semblance_eval(ctx, theta)
+        fctx.save_for_backward(theta)
+        return tt_semblance_eval(ctx, theta)
 
     @staticmethod
     def backward(fctx, gS):
-        _, dS = fctx.saved_tensors
+        theta, *kept = fctx.saved_tensors
+        if not kept or fctx.loads != fctx.tt.loads:
+            dS = tt_semblance_grad(fctx.tt, theta)[1]
+        elif fctx.plan == L.TT_GRAD_SUMS:
+            dS = _grad_sums(fctx.tt, theta, kept[0], fctx.stream)
+        else:
+            dS = kept[0]
         return None, gS.unsqueeze(-1) * dS, None
+
+
+def _grad_plan(ctx: Context, P: int):
+    """(plan, bytes of the sums) of a differentiated evaluation (include/tt.h)."""
+    plan, n_bytes = C.c_int32(), C.c_uint64()
+    _check(ctx.lib, ctx.handle, ctx.lib.tt_semblance_grad_plan(ctx.handle, P, C.byref(plan),
+                                                               C.byref(n_bytes)))
+    return plan.value, n_bytes.value
+
+
+def _eval_sums(ctx: Context, theta: torch.Tensor, sums: torch.Tensor, stream) -> torch.Tensor:
+    P = int(theta.shape[1])
+    tp = _ptr(theta, "theta", shape=(ctx.n_dom, P, ctx.D))
+    S = torch.empty((ctx.n_dom, P), dtype=torch.float32, device=theta.device)
+    _check(ctx.lib, ctx.handle, ctx.lib.tt_semblance_eval_sums(
+        ctx.handle, tp, P, S.data_ptr(), sums.data_ptr(), _stream(stream)))
+    return S
+
+
+def _grad_sums(ctx: Context, theta: torch.Tensor, sums: torch.Tensor, stream) -> torch.Tensor:
+    """theta as _eval_sums has checked it."""
+    dS = torch.empty_like(theta)
+    _check(ctx.lib, ctx.handle, ctx.lib.tt_semblance_grad_sums(
+        ctx.handle, theta.data_ptr(), theta.shape[1], sums.data_ptr(), dS.data_ptr(),
+        _stream(stream)))
+    return dS
 
 
 def semblance(ctx: Context, theta: torch.Tensor) -> torch.Tensor:

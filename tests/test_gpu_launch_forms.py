@@ -229,3 +229,49 @@ def test_gradient_of_infinite_energy(n_dom, P, sizes, op, w, ns, storage, bad):
         assert S.isnan().any() and G[S.isnan()].isnan().all()
     else:
         assert (S == 0).any() and not S.isnan().any() and not G.isnan().any()
+
+
+@pytest.mark.parametrize("n_dom,P,sizes,op,w,storage,ns,split,launches,same", [
+    (60, 2, (48,), 1, 5, "f32", 300, True, 1, True),          # the adjoint at once
+    (4001, 1, (600, 590), 1, 5, "f32", 300, True, 2, True),   # sums of clusters of 9
+    (4001, 1, (600, 590), 2, 8, "bf16", 300, True, 2, True),
+    (19000, 1, (150, 140), 1, 5, "f32", 2200, True, 2, True),  # of slices walked by 7 warps
+    (6333, 3, (250, 0), 1, 3, "bf16", 300, True, 2, True),
+    (60001, 1, (48,), 1, 5, "f32", 300, True, 2, True),       # of clusters of 2
+    (170000, 1, (60, 17), 1, 5, "bf16", 300, True, 2, False),  # of one block; K2 does not split
+    (117001, 1, (300,), 1, 1, "f32", 300, True, 2, True),
+    (300000, 1, (8,), 1, 5, "f32", 300, True, 2, True),       # too short: two launches
+    (312000, 1, (20,), 1, 5, "f32", 300, True, 2, True),      # too many pairs to split
+    (4001, 1, (600,), 1, 5, "f32", 300, False, 2, True)])
+def test_autograd_value_and_gradient(n_dom, P, sizes, op, w, storage, ns, split, launches, same):
+    """A differentiated call's value is tt_semblance_eval's bit for bit and costs
+    one launch while no backward comes; its gradient is tt_semblance_grad's bit for
+    bit wherever both split or neither does, and one of the same terms added in
+    another order elsewhere (the bound of test_split_gradient). A backward after a
+    reload is taken on the new traces."""
+    x, mid, off = _line(60, ns)
+    prob = _problem(n_dom, sizes, 60, ns, op, w)
+    ctx = tt.tt_ctx_create(x, mid, off, prob, None, storage=storage, device=dev())
+    tt.tt_ctx_set_option(ctx, "split", split)
+    th = to_dev(random_theta(n_dom, P, *BOUNDS[op], 5)).requires_grad_()
+    gS = torch.rand((n_dom, P), device=dev())
+    E = tt.tt_semblance_eval(ctx, th.detach())
+    tt.tt_ctx_stats(ctx, reset=True)
+    S = tt.semblance(ctx, th)
+    assert tt.tt_ctx_stats(ctx)["launches"] == 1 and torch.equal(S.detach(), E)
+    S.backward(gS, retain_graph=True)
+    assert tt.tt_ctx_stats(ctx)["launches"] == launches
+    G = tt.tt_semblance_grad(ctx, th.detach())[1] * gS.unsqueeze(-1)
+
+    def check(G):
+        if same:
+            assert torch.equal(th.grad, G)
+        scale = G.abs().flatten(0, 1).median(0).values
+        assert ((th.grad - G).abs() <= 1e-3 * (G.abs() + scale)).all()
+
+    check(G)
+    th.grad = None
+    tt.tt_ctx_load_traces(ctx, torch.from_numpy(x[::-1].copy()))
+    S.backward(gS)
+    check(tt.tt_semblance_grad(ctx, th.detach())[1] * gS.unsqueeze(-1))
+    ctx.close()
