@@ -64,6 +64,7 @@ tt::EvalArgs tt_ctx::eval_args(const float* theta, int P, float* S) const {
   a.n_sm = n_sm;
   a.n_groups = n_groups;
   a.mean_ap = n_dom > 0 ? float(sum_N / n_dom) : 0.f;
+  a.max_ap = max_N;
   a.queue = queue;
   return a;
 }
@@ -572,7 +573,8 @@ extern "C" tt_status tt_ctx_create(tt_ctx** out, const tt_gathers* ga, const tt_
     TRY(cudaMemcpyAsync(c->dom_group, pr->dom_group, size_t(c->n_dom) * 4,
                         cudaMemcpyDeviceToDevice, s), "copy groups");
   }
-  // sum over domains of the aperture size (for the trace-evaluation counter)
+  // sum over domains of the aperture size (for the trace-evaluation counter and
+  // the launch rules) and the largest
   if (c->n_dom > 0) {
     std::vector<int> hp(size_t(c->n_groups) + 1), hg(size_t(c->n_dom));
     TRY(cudaMemcpyAsync(hp.data(), pr->ap_ptr, hp.size() * 4, cudaMemcpyDeviceToHost, s),
@@ -581,8 +583,14 @@ extern "C" tt_status tt_ctx_create(tt_ctx** out, const tt_gathers* ga, const tt_
         "read groups");
     TRY(cudaStreamSynchronize(s), "sync");
     double sn = 0;
-    for (int g : hg) sn += hp[g + 1] - hp[g];
+    int mn = 0;
+    for (int g : hg) {
+      const int n = hp[g + 1] - hp[g];
+      sn += n;
+      mn = std::max(mn, n);
+    }
     c->sum_N = sn;
+    c->max_N = mn;
   }
   // search scratch
   if (c->has_cfg) {

@@ -60,7 +60,12 @@ cudaError_t launch_split(EvalArgs& a, long long units, bool mv, cudaStream_t s) 
   // 56 take to come and go: 48 traces 118 / 258 units 8.7 / 10.4 us against
   // 10.5 / 18.5 us, 144 traces 258 units 18.6 against 22.8 us; 336 traces 118 /
   // 258 units 20.7 / 34.9 us against 16.7 / 31.1 us
-  if (B == kSplitSmallBlocks && a.mean_ap <= 0.6f * float(units)) {
+  // The launch ends with its longest aperture, which eight times fewer warps walk:
+  // 300 units of 40 traces, one of 2000: 121 us against 25 us; ten of 240 / 320 20.6 /
+  // 25.8 against 22.3 / 22.8; 160 units of 40, ten of 120 / 160 14.1 / 16.3 against
+  // 12.6 / 13.3; 300 units of 150, twenty of 250 26.7 against 30.6.
+  if (B == kSplitSmallBlocks && a.mean_ap <= 0.6f * float(units) &&
+      float(a.max_ap) <= 0.7f * float(units) + 0.5f * a.mean_ap) {
     const KFn fn = pick(sk::kKindShort, a, mv);
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = sk::short_smem_bytes(kSplitSmallBlocks, a.W, bf);
@@ -250,13 +255,24 @@ size_t grad_sums_bytes(const EvalArgs& a) {
 // block are nearly full: DE 32 x 30 on 38 / 150 / 300 units of 48 traces 144 /
 // 134 / 173 us against 291 / 302 / 344 us stepwise, of 144 traces 253 / 267 /
 // 370 against 289 / 504 / 525, of 336 traces 446 / 665 / 799 against 341 / 672
-// / 1122, of 1008 traces 1258 / 1898 / 2164 against 602 / 1352 / 2297.
+// / 1122, of 1008 traces 1258 / 1898 / 2164 against 602 / 1352 / 2297. A block
+// holds 64 / NP whole domains, so that populations of 33 to 60 members fill it
+// less and a launch may need a second wave: up to 120 traces then (NP 33, 589
+// blocks for 304 units, 48 / 120 / 160 traces 319 / 630 / 769 us against 393 / 647
+// / 749 us). A search ends with its longest aperture, by seven warps where the
+// stepwise launch has 56: 76 domains, mean 66 to 70 traces, longest 180 / 240 / 600
+// 295 / 356 / 781 us against 287 / 299 / 352 us; 300 of mean 22, longest 250 / 310
+// 365 / 472 against 378 / 380; 600 of mean 99 to 110, longest 400 / 450 798 / 1023
+// against 838 / 864.
 bool fused_search_fits(const EvalArgs& a) {
   const long long units = ((long long)a.n_dom * a.P + 63) / 64;
   if (!a.split || a.P > 64 || a.dom_map || units > (long long)a.n_sm * kSplitSmallPerSm)
     return false;
-  return a.mean_ap <= 160.f ||
-         (a.mean_ap <= 1.5f * float(units) && 64 / a.P * a.P * 6 >= 64 * 5);
+  const int per = 64 / a.P;
+  const long long blocks = (a.n_dom + per - 1) / per;
+  if (float(a.max_ap) > a.mean_ap + 110.f + 0.75f * float(units)) return false;
+  return a.mean_ap <= (blocks > 2ll * a.n_sm ? 120.f : 160.f) ||
+         (a.mean_ap <= 1.5f * float(units) && per * a.P * 6 >= 64 * 5);
 }
 
 cudaError_t launch_fused_search(const EvalArgs& a, const DeArgs& de, const FusedArgs& f,
@@ -269,8 +285,9 @@ cudaError_t launch_fused_search(const EvalArgs& a, const DeArgs& de, const Fused
     case TT_OP_CRS: fn = sk::pick_fused<TT_OP_CRS>(a.storage, a.W, mv); break;
     case TT_OP_FOCRS: fn = sk::pick_fused<TT_OP_FOCRS>(a.storage, a.W, mv); break;
   }
-  if (!fn || a.P > 64) return cudaErrorInvalidValue;
   const int B = split_blocks(((long long)a.n_dom * a.P + 63) / 64, a.n_sm);
+  // the kernel adds kSplitSmallBlocks or kSplitTinyBlocks sets, no fewer
+  if (!fn || a.P > 64 || B < kSplitSmallBlocks) return cudaErrorInvalidValue;
   const int per = 64 / a.P;
   const bool bf = a.storage == TT_STORE_BF16;
   const size_t smem = sk::short_smem_bytes(B, a.W, bf);

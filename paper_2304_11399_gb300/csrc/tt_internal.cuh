@@ -70,6 +70,7 @@ struct EvalArgs {
   double* sums_Ed;
   int n_groups;             // aperture groups of the context
   float mean_ap;            // mean aperture size over the context's domains
+  int max_ap;               // and the largest
 };
 
 cudaError_t launch_semblance(const EvalArgs& a, cudaStream_t s);
@@ -261,6 +262,7 @@ struct tt_ctx {
   std::string err;
   // counters and optional event timing of semblance launches
   double sum_N = 0;         // sum over domains of the aperture size
+  int max_N = 0;            // the largest
   unsigned long long n_launch = 0, n_sem = 0, n_timed = 0;
   double trace_evals = 0;
   bool profiling = false;

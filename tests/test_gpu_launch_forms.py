@@ -275,3 +275,49 @@ def test_autograd_value_and_gradient(n_dom, P, sizes, op, w, storage, ns, split,
     S.backward(gS)
     check(tt.tt_semblance_grad(ctx, th.detach())[1] * gS.unsqueeze(-1))
     ctx.close()
+
+
+@pytest.mark.parametrize("op,w,storage,ns", [(1, 5, "f32", 300), (0, 3, "f32", 2200),
+                                             (2, 8, "bf16", 300), (1, 4, "bf16", 2200)])
+def test_uneven_slices_walked_by_one_warp_or_eight(op, w, storage, ns):
+    """One unit per SM and two: the same 56 slices of apertures of 0, 1 and up to
+    1.39 traces per SM, by a warp each at one unit (mean above 0.6 traces a unit),
+    by a warp for eight at two (mean below that, largest below 0.7 and half the
+    mean)."""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    sizes = [int(f * n_sm) for f in (1.3, 1.39, 1.0, 0.65, 0.8)] + [0, 1]
+    n_dom = 8 * n_sm
+    x, mid, off = _line(60, ns)
+    prob = _problem(n_dom, sizes, 60, ns, op, w)
+    mean = np.diff(prob.ap_ptr)[prob.dom_group].mean()
+    assert 0.6 * n_sm < mean < 1.2 * n_sm and max(sizes) < 1.4 * n_sm + 0.5 * mean
+    bounds = BOUNDS[op] if op else ((1 / 4500 ** 2,), (1 / 1400 ** 2,))
+    th = to_dev(random_theta(n_dom, 16, *bounds, 7))
+    ctx = tt.tt_ctx_create(x, mid, off, prob, None, storage=storage, device=dev())
+    a = tt.tt_semblance_eval(ctx, th[:, :8].contiguous())
+    b = tt.tt_semblance_eval(ctx, th)
+    ctx.close()
+    assert torch.equal(a, b[:, :8])
+    if storage == "f32":
+        ref = oracle.semblance.semblance_many(x, mid, off, prob, th[:, :1].cpu().numpy())
+        assert np.max(np.abs(a[:, :1].cpu().numpy() - ref)) <= 1e-5
+
+
+@pytest.mark.parametrize("sizes,np_", [((48,) * 30 + (900,), 32), ((150,), 33)])
+def test_stepwise_where_fused_is_slower(sizes, np_):
+    """A long aperture among short ones, and a second wave of half-filled blocks:
+    the search runs step by step (as many launches as while it is timed)."""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    n_dom = 2 * n_sm + 1
+    x, mid, off = _line(60, 300)
+    prob = _problem(n_dom, sizes, 60, 300)
+    ctx = tt.tt_ctx_create(x, mid, off, prob, _cfg(1, np_, 3), device=dev())
+    tt.tt_ctx_set_option(ctx, "search_graph", False)
+    tt.tt_ctx_stats(ctx, reset=True)
+    th, S, _ = tt.tt_search(ctx)
+    few = tt.tt_ctx_stats(ctx, reset=True)
+    tt.tt_ctx_profile(ctx, True)
+    th1, S1, _ = tt.tt_search(ctx)
+    assert few["launches"] == tt.tt_ctx_stats(ctx)["launches"]
+    ctx.close()
+    assert torch.equal(th, th1) and torch.equal(S, S1)
