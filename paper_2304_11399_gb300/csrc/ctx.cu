@@ -62,7 +62,7 @@ tt::EvalArgs tt_ctx::eval_args(const float* theta, int P, float* S) const {
   a.split = split ? 1 : 0;
   a.split_blocks = 1;
   a.n_sm = n_sm;
-  a.n_groups = n_groups;
+  a.n_runs = n_runs;
   a.mean_ap = n_dom > 0 ? float(sum_N / n_dom) : 0.f;
   a.max_ap = max_N;
   a.queue = queue;
@@ -574,7 +574,7 @@ extern "C" tt_status tt_ctx_create(tt_ctx** out, const tt_gathers* ga, const tt_
                         cudaMemcpyDeviceToDevice, s), "copy groups");
   }
   // sum over domains of the aperture size (for the trace-evaluation counter and
-  // the launch rules) and the largest
+  // the launch rules), the largest, and the runs of domains of one group
   if (c->n_dom > 0) {
     std::vector<int> hp(size_t(c->n_groups) + 1), hg(size_t(c->n_dom));
     TRY(cudaMemcpyAsync(hp.data(), pr->ap_ptr, hp.size() * 4, cudaMemcpyDeviceToHost, s),
@@ -583,14 +583,17 @@ extern "C" tt_status tt_ctx_create(tt_ctx** out, const tt_gathers* ga, const tt_
         "read groups");
     TRY(cudaStreamSynchronize(s), "sync");
     double sn = 0;
-    int mn = 0;
+    int mn = 0, runs = 0, last = -1;
     for (int g : hg) {
       const int n = hp[g + 1] - hp[g];
       sn += n;
       mn = std::max(mn, n);
+      runs += g != last;
+      last = g;
     }
     c->sum_N = sn;
     c->max_N = mn;
+    c->n_runs = runs;
   }
   // search scratch
   if (c->has_cfg) {

@@ -201,14 +201,16 @@ cudaError_t launch_stack(const EvalArgs& a, float* out, cudaStream_t s) {
   if (a.n_dom == 0) return cudaSuccess;
   if (a.P != 1) return cudaErrorInvalidValue;
   const bool mv = a.umax > float(kDirectMax);
-  // One lane per domain where consecutive domains mostly share an aperture: 4
-  // domains per group on average already win (2000 groups of 4, 1008 traces:
-  // 29 us against 42 us with a warp per domain; of 1500: below). One warp per
+  // One lane per domain where consecutive domains mostly share an aperture: runs
+  // of 4 domains of a group on average already win (2000 groups of 4, 1008 traces:
+  // 29 us against 42 us with a warp per domain; of 1500: below). Groups whose
+  // domains are scattered (200 groups x 1500 with the group changing at every
+  // domain: 1734 us against 761 us) keep the warp per domain. One warp per
   // sum until the launch has 16 groups of 32 domains per SM, then 8 sums per
   // warp (20 / 60 / 200 CMPs x 1500 samples, 1008 traces, one sum a warp 36 /
   // 87 / 305 us, eight 45 / 88 / 241 us, a warp per domain 93 / 265 / 843 us).
   const long long groups32 = ((long long)a.n_dom + 31) / 32;
-  const int rows = a.n_dom < 4ll * a.n_groups ? 0 : groups32 < 16ll * a.n_sm ? 1 : 8;
+  const int rows = a.n_dom < 4ll * a.n_runs ? 0 : groups32 < 16ll * a.n_sm ? 1 : 8;
   sk::SFn fn = nullptr;
   switch (a.op) {
     case TT_OP_CMP: fn = sk::pick_stack<TT_OP_CMP>(a.storage, mv, rows); break;

@@ -68,7 +68,7 @@ struct EvalArgs {
   // gradient launch starts from them instead of a first pass; NULL: neither.
   float* sums;
   double* sums_Ed;
-  int n_groups;             // aperture groups of the context
+  int n_runs;               // runs of consecutive domains of one group
   float mean_ap;            // mean aperture size over the context's domains
   int max_ap;               // and the largest
 };
@@ -263,6 +263,7 @@ struct tt_ctx {
   // counters and optional event timing of semblance launches
   double sum_N = 0;         // sum over domains of the aperture size
   int max_N = 0;            // the largest
+  int n_runs = 0;           // runs of consecutive domains of one group
   unsigned long long n_launch = 0, n_sem = 0, n_timed = 0;
   double trace_evals = 0;
   bool profiling = false;
