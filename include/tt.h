@@ -175,25 +175,18 @@ tt_status tt_semblance_grad(tt_ctx* ctx, const float* theta, int32_t P, float* S
                             void* stream);
 
 /* A value whose gradient may be asked for later, or never (the autograd use of
- * the two calls above). tt_semblance_grad_plan says how a launch of P vectors
- * per domain is best run with the context's present options:
- *  TT_GRAD_SEPARATE  tt_semblance_eval, later tt_semblance_grad.
- *  TT_GRAD_TOGETHER  tt_semblance_grad at once (a launch too small for the
- *                    second pass to show beside its issue); its S is
- *                    tt_semblance_eval's bit for bit.
- *  TT_GRAD_SUMS      tt_semblance_eval_sums, which is tt_semblance_eval and
- *                    keeps every pair's sums in `sums` (device memory of the
- *                    caller, *bytes long, 16-byte aligned), later
- *                    tt_semblance_grad_sums with the same theta and P, on the
- *                    same traces: the gradient's second pass alone.
- * *bytes is 0 for the first two. TT_ERR_INVALID_ARG for NULL arrays, and from
- * tt_semblance_eval_sums where the plan is another. */
-typedef enum {
-  TT_GRAD_SEPARATE = 0,
-  TT_GRAD_TOGETHER = 1,
-  TT_GRAD_SUMS = 2
-} tt_grad_plan;
-tt_status tt_semblance_grad_plan(tt_ctx* ctx, int32_t P, int32_t* plan, uint64_t* bytes);
+ * the two calls above). tt_semblance_sums_size says how a launch of P vectors
+ * per domain is best run with the context's present options, by *bytes:
+ *  > 0  tt_semblance_eval_sums, which is tt_semblance_eval and keeps every
+ *       pair's sums in `sums` (device memory of the caller, *bytes long, 16-byte
+ *       aligned), later tt_semblance_grad_sums with the same theta and P on the
+ *       same traces: the gradient's second pass alone;
+ *  0    tt_semblance_eval, later tt_semblance_grad;
+ *  -1   tt_semblance_grad at once (a launch too small for the second pass to
+ *       show beside its issue); its S is tt_semblance_eval's bit for bit.
+ * TT_ERR_INVALID_ARG for NULL arrays, and from tt_semblance_eval_sums where
+ * *bytes is not positive. */
+tt_status tt_semblance_sums_size(tt_ctx* ctx, int32_t P, int64_t* bytes);
 tt_status tt_semblance_eval_sums(tt_ctx* ctx, const float* theta, int32_t P, float* S, void* sums,
                                  void* stream);
 tt_status tt_semblance_grad_sums(tt_ctx* ctx, const float* theta, int32_t P, const void* sums,

@@ -13,7 +13,6 @@ TT_OP_CMP, TT_OP_CRS, TT_OP_FOCRS = 0, 1, 2
 TT_OPT_KERNEL, TT_OPT_BLOCK, TT_OPT_SEARCH_GRAPH, TT_OPT_SPLIT = 1, 2, 3, 4
 TT_OPT_SPLIT_MAX_PAIRS, TT_OPT_SM_COUNT, TT_OPT_MEMBER_ORDER = 5, 6, 7
 TT_KERNEL_PACKED, TT_KERNEL_PERSISTENT, TT_KERNEL_SCALAR = 1, 2, 3
-TT_GRAD_SEPARATE, TT_GRAD_TOGETHER, TT_GRAD_SUMS = 0, 1, 2
 TT_N_TUNE_CANDIDATES = 6
 TUNE_CANDIDATES = [("packed", 256), ("packed", 128), ("persistent", 256), ("persistent", 128),
                    ("scalar", 256), ("scalar", 128)]
@@ -78,7 +77,7 @@ SIGNATURES = {
     "tt_ctx_destroy": (None, [P]),
     "tt_semblance_eval": (I32, [P, P, I32, P, P]),
     "tt_semblance_grad": (I32, [P, P, I32, P, P, P]),
-    "tt_semblance_grad_plan": (I32, [P, I32, C.POINTER(I32), C.POINTER(C.c_uint64)]),
+    "tt_semblance_sums_size": (I32, [P, I32, C.POINTER(C.c_int64)]),
     "tt_semblance_eval_sums": (I32, [P, P, I32, P, P, P]),
     "tt_semblance_grad_sums": (I32, [P, P, I32, P, P, P]),
     "tt_stack": (I32, [P, P, P, P]),

@@ -239,18 +239,13 @@ cudaError_t launch_semblance_grad(const EvalArgs& a, cudaStream_t s) { return la
 // and 301 us, which is host time). What the evaluation does not split, or holds
 // apertures too short for split gradients, is evaluated and differentiated by
 // launches of their own.
-int grad_plan(const EvalArgs& a) {
+long long grad_sums_bytes(const EvalArgs& a) {
   const long long n = (long long)a.n_dom * a.P, units = (n + 63) / 64;
   if (!a.split || n == 0 || units >= (long long)a.n_sm * kSplitUnitsPerSm || a.mean_ap < 16.f)
-    return TT_GRAD_SEPARATE;
-  return double(n) * a.mean_ap <= kGradTogetherMax && grad_split(a, units) ? TT_GRAD_TOGETHER
-                                                                           : TT_GRAD_SUMS;
-}
-
-size_t grad_sums_bytes(const EvalArgs& a) {
-  const size_t units = ((size_t)a.n_dom * a.P + 63) / 64;
-  return a.storage == TT_STORE_BF16 ? units * sk::split_set_bytes<__nv_bfloat16>(a.W)
-                                    : units * sk::split_set_bytes<float>(a.W);
+    return 0;
+  if (double(n) * a.mean_ap <= kGradTogetherMax && grad_split(a, units)) return -1;
+  return units * (long long)(a.storage == TT_STORE_BF16 ? sk::split_set_bytes<__nv_bfloat16>(a.W)
+                                                        : sk::split_set_bytes<float>(a.W));
 }
 
 // Apertures of up to 160 traces, or of 1.5 per unit where the 64 slots of a
@@ -388,14 +383,11 @@ extern "C" tt_status tt_semblance_grad(tt_ctx* ctx, const float* theta, int32_t 
                        "semblance gradient launch");
 }
 
-extern "C" tt_status tt_semblance_grad_plan(tt_ctx* ctx, int32_t P, int32_t* plan,
-                                            uint64_t* bytes) {
+extern "C" tt_status tt_semblance_sums_size(tt_ctx* ctx, int32_t P, int64_t* bytes) {
   if (!ctx) return tt_fail(nullptr, TT_ERR_INVALID_ARG, "ctx is NULL");
   if (P < 1) return tt_fail(ctx, TT_ERR_INVALID_ARG, "P must be >= 1");
-  if (!plan || !bytes) return tt_fail(ctx, TT_ERR_INVALID_ARG, "plan or bytes is NULL");
-  const tt::EvalArgs a = ctx->eval_args(nullptr, P, nullptr);
-  *plan = tt::grad_plan(a);
-  *bytes = *plan == TT_GRAD_SUMS ? tt::grad_sums_bytes(a) : 0;
+  if (!bytes) return tt_fail(ctx, TT_ERR_INVALID_ARG, "bytes is NULL");
+  *bytes = tt::grad_sums_bytes(ctx->eval_args(nullptr, P, nullptr));
   return TT_OK;
 }
 
@@ -417,7 +409,7 @@ extern "C" tt_status tt_semblance_eval_sums(tt_ctx* ctx, const float* theta, int
   if (P < 1) return tt_fail(ctx, TT_ERR_INVALID_ARG, "P must be >= 1");
   if (!theta || !S || !sums) return tt_fail(ctx, TT_ERR_INVALID_ARG, "NULL array");
   tt::EvalArgs a = ctx->eval_args(theta, P, S);
-  if (tt::grad_plan(a) != TT_GRAD_SUMS)
+  if (tt::grad_sums_bytes(a) <= 0)
     return tt_fail(ctx, TT_ERR_INVALID_ARG, "this launch keeps no sums");
   set_sums(a, sums);
   return tt_cuda_check(ctx, ctx->semblance(a, static_cast<cudaStream_t>(stream), false),

@@ -75,8 +75,7 @@ struct EvalArgs {
 
 cudaError_t launch_semblance(const EvalArgs& a, cudaStream_t s);
 cudaError_t launch_semblance_grad(const EvalArgs& a, cudaStream_t s);
-int grad_plan(const EvalArgs& a);          // TT_GRAD_*
-size_t grad_sums_bytes(const EvalArgs& a); // of a TT_GRAD_SUMS launch
+long long grad_sums_bytes(const EvalArgs& a);  // what tt_semblance_sums_size says
 // Members of each domain of theta (a.theta, a.P <= 256, no domain map) sorted
 // by window position: parameters to theta_out, original slots to slots
 // ([n_dom][P]); evaluate theta_out with slots as the scatter map.

@@ -401,7 +401,7 @@ class SemblanceFn(torch.autograd.Function):
     """S(theta), as tt_semblance_eval gives it, with the hand-written adjoint
     kernel as its backward. ``adjoint`` says whether a backward can follow
     (default: whether theta requires a gradient); without one the call is
-    tt_semblance_eval. With one it runs as tt_semblance_grad_plan says: the
+    tt_semblance_eval. With one it runs as tt_semblance_sums_size says: the
     evaluation keeps each pair's sums (2w + 2 floats a pair, held until the graph
     is freed) and the backward is the adjoint's second pass alone; a call of a few
     microseconds of device time runs the adjoint at once and keeps dS/dtheta; any
@@ -418,38 +418,34 @@ class SemblanceFn(torch.autograd.Function):
             return tt_semblance_eval(ctx, theta)
         if theta.dim() != 3:
             raise ValueError("theta must be [n_dom, P, D]")
-        fctx.tt, fctx.loads = ctx, ctx.loads
-        fctx.plan, n_bytes = _grad_plan(ctx, int(theta.shape[1]))
-        if fctx.plan == L.TT_GRAD_SUMS:
-            sums = torch.empty((n_bytes,), dtype=torch.uint8, device=theta.device)
-            fctx.save_for_backward(theta, sums)
-            fctx.stream = torch.cuda.current_stream()  # which autograd's backward runs on too
-            return _eval_sums(ctx, theta, sums, fctx.stream)
-        if fctx.plan == L.TT_GRAD_TOGETHER:
+        n_bytes = C.c_int64()
+        _check(ctx.lib, ctx.handle, ctx.lib.tt_semblance_sums_size(
+            ctx.handle, theta.shape[1], C.byref(n_bytes)))
+        if n_bytes.value < 0:
+            fctx.call = ctx, ctx.loads, None
             S, dS = tt_semblance_grad(ctx, theta)
             fctx.save_for_backward(theta, dS)
             return S if ctx.storage == "f32" else tt_semblance_eval(ctx, theta)
-        fctx.save_for_backward(theta)
-        return tt_semblance_eval(ctx, theta)
+        # autograd's backward runs on this stream too
+        fctx.call = ctx, ctx.loads, torch.cuda.current_stream()
+        if n_bytes.value == 0:
+            fctx.save_for_backward(theta)
+            return tt_semblance_eval(ctx, theta)
+        sums = torch.empty((n_bytes.value,), dtype=torch.uint8, device=theta.device)
+        fctx.save_for_backward(theta, sums)
+        return _eval_sums(ctx, theta, sums, fctx.call[2])
 
     @staticmethod
     def backward(fctx, gS):
         theta, *kept = fctx.saved_tensors
-        if not kept or fctx.loads != fctx.tt.loads:
-            dS = tt_semblance_grad(fctx.tt, theta)[1]
-        elif fctx.plan == L.TT_GRAD_SUMS:
-            dS = _grad_sums(fctx.tt, theta, kept[0], fctx.stream)
-        else:
+        ctx, loads, stream = fctx.call
+        if not kept or loads != ctx.loads:
+            dS = tt_semblance_grad(ctx, theta)[1]
+        elif stream is None:
             dS = kept[0]
+        else:
+            dS = _grad_sums(ctx, theta, kept[0], stream)
         return None, gS.unsqueeze(-1) * dS, None
-
-
-def _grad_plan(ctx: Context, P: int):
-    """(plan, bytes of the sums) of a differentiated evaluation (include/tt.h)."""
-    plan, n_bytes = C.c_int32(), C.c_uint64()
-    _check(ctx.lib, ctx.handle, ctx.lib.tt_semblance_grad_plan(ctx.handle, P, C.byref(plan),
-                                                               C.byref(n_bytes)))
-    return plan.value, n_bytes.value
 
 
 def _eval_sums(ctx: Context, theta: torch.Tensor, sums: torch.Tensor, stream) -> torch.Tensor:
