@@ -170,7 +170,9 @@ tt_status tt_semblance_eval(tt_ctx* ctx, const float* theta, int32_t P, float* S
 /* Semblance and its gradient dS/dtheta (an addition to the paper's method,
  * used to polish the DE winner) by the adjoint of the interpolation and
  * traveltime: inside an interpolation cell da_ik/du_i = x_i[j+k+1]-x_i[j+k].
- * theta [n_dom][P][D], S [n_dom][P], dS [n_dom][P][D]. */
+ * theta [n_dom][P][D], S [n_dom][P], dS [n_dom][P][D]. A launch that is split
+ * (TT_OPT_SPLIT) sums as tt_semblance_eval does; one that is not adds the whole
+ * aperture's energy in FP32, also for BF16-stored traces. */
 tt_status tt_semblance_grad(tt_ctx* ctx, const float* theta, int32_t P, float* S, float* dS,
                             void* stream);
 
@@ -361,8 +363,9 @@ tt_status tt_ctx_probe_l1(tt_ctx* ctx, int32_t iters, double* bytes, void* strea
  *                 within 1e-5 of the exact semblance). Searches of few domains
  *                 with short apertures run all generations between exchanges
  *                 in one launch, with the same sums. Gradient evaluations are
- *                 split too (tt_semblance_grad; not inside the polish, whose
- *                 iterates are compared by their S). 0: never split.
+ *                 split too (tt_semblance_grad; not the gradients inside the
+ *                 polish, whose iterates are compared by their S; its last
+ *                 iterate is evaluated like any population). 0: never split.
  *  TT_OPT_MEMBER_ORDER  1: before each generation's evaluation inside
  *                 tt_search / tt_search_slab (NP <= 256), the members of
  *                 every domain are put in the order of their window position

@@ -26,7 +26,11 @@ tt_status polish_impl(tt_ctx* c, const float* theta_in, float* theta_out, float*
   for (int k = 0; k < steps; ++k) {
     tt::EvalArgs a = c->eval_args(c->pol_th, 1, c->pol_S);
     a.dS = c->pol_g;
-    a.split = 0;  // S of successive iterates is compared: one summation order for every launch
+    // The iterates' S are compared: unsplit, so that their sums are of one order
+    // whatever the number of domains. The last iterate's S, below, is a plain
+    // evaluation: split by launch size, with BF16 storage's FP64 energy, so that
+    // it wins or loses by rounding where it lies within rounding of the best.
+    a.split = 0;
     st = tt_cuda_check(c, c->semblance(a, s, true), "polish gradient");
     if (st != TT_OK) return st;
     st = tt_cuda_check(c, c->counted(tt::launch_polish_update(n, D, c->pol_th, c->pol_g, c->pol_S,
