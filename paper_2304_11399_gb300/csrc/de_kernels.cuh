@@ -163,9 +163,10 @@ __device__ inline void jade_select(const DeArgs& a, int d, uint32_t gd, uint32_t
         slot = int(__umulhi(w.x, uint32_t(NP)));
       }
       const unsigned same = __match_any_sync(m, slot);
-      if (31 - __clz(same) == lane)
-        #pragma unroll
-      for (int q = 0; q < D; ++q) arc[slot * D + q] = p.pop[i * D + q];
+      if (31 - __clz(same) == lane) {
+#pragma unroll
+        for (int q = 0; q < D; ++q) arc[slot * D + q] = p.pop[i * D + q];
+      }
     }
     for (unsigned mm = m; mm; mm &= mm - 1) {
       const int j = __ffs(mm) - 1;

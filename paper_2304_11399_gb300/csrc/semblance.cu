@@ -101,11 +101,11 @@ cudaError_t launch_split(EvalArgs& a, long long units, bool mv, cudaStream_t s) 
 
 // Split gradient launches: where forward launches split (their sums then agree
 // bit for bit, and so does S), with apertures of 256 traces or more (1008
-// traces: 24 / 938 / 4688 units 28 / 474 / 1963 us against 740 / 839 / 2126 us
-// with one pair per thread), with shorter ones down to 16 traces while the
-// launch has fewer than 16 units per SM (144 traces: 469 units 75 us against
-// 98 us, 4688 units 322 us against 307 us; 48 traces: 16 units 18 us against 50
-// us, 9375 units 284 us against 217 us).
+// traces: 24 / 282 / 938 / 4688 units 28 / 189 / 473 / 1962 us against 319 / 374 /
+// 572 / 2217 us with one pair per thread), with shorter ones down to 16 traces
+// while the launch has fewer than 16 units per SM (144 traces: 469 units 60 us
+// against 67 us, 4688 units 322 us against 307 us; 48 traces: 16 units 16 us
+// against 19 us, 9375 units 284 us against 217 us).
 bool grad_split(const EvalArgs& a, long long units) {
   return a.split && units < (long long)a.n_sm * kSplitUnitsPerSm &&
          (a.mean_ap >= 256.f || (a.mean_ap >= 16.f && units < 16ll * a.n_sm));
@@ -116,10 +116,11 @@ bool grad_split(const EvalArgs& a, long long units) {
 // 33 us to issue (4 million: 52 to 59 us).
 constexpr double kGradTogetherMax = 2097152.0;
 
-// The cluster has the forward launch's B blocks (1008 traces, clusters of 1 / 2
-// / 4 / 8: 24 units 115 / 66 / 38 / 28 us, 282 units 308 / 235 / 207 / 217 us,
-// 938 units 647 / 562 / 577 / 680 us, at two blocks per SM: the rule's 9, 7 and
-// 2 lie near the best).
+// The cluster has the forward launch's B blocks, 9, 7, 2 or 1, so that S agrees
+// with it (1008 traces, clusters of 1 / 2 / 4 / 7 / 8 / 9: 24 units 107 / 61 / 36 /
+// 32 / 27 / 27 us, 282 units 290 / 217 / 176 / 189 / 185 / 189 us, 938 units 560 /
+// 473 / 468 / 574 / 565 / 591 us, 4688 units 1964 / 1972 / 2157 / 2767 / 2740 / 2888
+// us: the rule's 9, 7, 2 and 1 lie within 8% of the best).
 cudaError_t launch_grad_split(const EvalArgs& a, long long units, bool mv, cudaStream_t s) {
   const KFn fn = pick(sk::kKindGradSplit, a, mv);
   if (!fn) return cudaErrorInvalidValue;
@@ -367,8 +368,8 @@ extern "C" tt_status tt_stack(tt_ctx* ctx, const float* theta, float* out, void*
   if (!ctx) return tt_fail(nullptr, TT_ERR_INVALID_ARG, "ctx is NULL");
   if (ctx->n_dom > 0 && (!theta || !out)) return tt_fail(ctx, TT_ERR_INVALID_ARG, "NULL array");
   tt::EvalArgs a = ctx->eval_args(theta, 1, nullptr);
-  return tt_cuda_check(ctx, ctx->counted(tt::launch_stack(a, out, static_cast<cudaStream_t>(stream))),
-                       "stack launch");
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  return tt_cuda_check(ctx, ctx->counted(tt::launch_stack(a, out, s)), "stack launch");
 }
 
 extern "C" tt_status tt_semblance_grad(tt_ctx* ctx, const float* theta, int32_t P, float* S,

@@ -538,7 +538,8 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 4) k_semblance_split(const E
   const int sets = S + (B > 1 && !PULL ? B : 0);
   float* part = reinterpret_cast<float*>(part_Ed + (Chunk<T>::kF64 ? sets * 64 : 0));
   float* recv = part + S * R * 64;  // [B][R][64], in the cluster's first block
-  if (B > 1 && !PULL) cluster_arrive_relaxed();  // met by cluster_wait below: every block has started
+  // met by cluster_wait below: every block has started
+  if (B > 1 && !PULL) cluster_arrive_relaxed();
   const long long q0 = unit * 64 + lane, q1 = q0 + 32;
   Lane L0, L1;
   const bool v0 = lane_setup<OP, true>(a, q0, L0);
@@ -1197,10 +1198,11 @@ __global__ void __launch_bounds__(128) k_semblance_grad(const EvalArgs a) {
 // (blocks in order); the cluster barriers take the place of a second launch.
 // The gradient usually has one pair per domain, so that a thread per pair
 // leaves a few warps per SM, each waiting on 1008 x 2 dependent window loads:
-// 60,000 CRS domains, 1008 traces, w = 5: 962 us, now 474 us; 1500 domains 835
-// us, now 28 us. Three blocks per SM (80 registers) hide more load latency
-// than two (102 registers: 562 us); it stays bound by its window loads (two
-// passes at K1's rate).
+// 60,000 CRS domains, 1008 traces, w = 5: 880 us (572 us with six entries in
+// flight), now 473 us; 1500 domains 700 us (319 us), now 28 us. Three blocks per
+// SM (80 registers) hide more load latency than two (540 us); it stays bound by
+// its window loads (two passes at K1's rate). From sums that the evaluation kept
+// (a.sums) it is the second pass alone.
 constexpr int kGradWarps = 8;
 
 // shared memory of a block: FP64 energies [kGradWarps + 1][64]; rows of 64
@@ -1301,7 +1303,8 @@ __global__ void __launch_bounds__(32 * kGradWarps, 3) k_semblance_grad_split(con
     if (a.sums)
       t = a.sums[unit * (R * 64) + i];
     else
-      for (int b = 0; b < B; ++b) t = __fadd_rn(t, B > 1 ? cl.map_shared_rank(blk, b)[i] : blk[i]);
+      for (int b = 0; b < B; ++b)
+        t = __fadd_rn(t, B > 1 ? cl.map_shared_rank(blk, b)[i] : blk[i]);
     tot[i] = t;
   }
   __syncthreads();
