@@ -120,6 +120,25 @@ def test_split_gradient(n_dom, P, sizes, op, w, storage, ns):
         assert rS is None or np.max(np.abs(S.cpu().numpy() - rS)) <= 1e-5
 
 
+def test_split_gradient_of_one_block():
+    """12 units per SM and one pair more: a unit's aperture in one block (B = 1),
+    against the unsplit form, with the bounds of test_split_gradient (n = 900)."""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    n_dom = 12 * n_sm * 64 + 1
+    x, mid, off = _line(60, 300)
+    ctx = tt.tt_ctx_create(x, mid, off, _problem(n_dom, (300,), 60, 300, w=1), None,
+                           device=dev())
+    th = to_dev(random_theta(n_dom, 1, *BOUNDS[1], 5))
+    S, G = tt.tt_semblance_grad(ctx, th)
+    assert torch.equal(S, tt.tt_semblance_eval(ctx, th))
+    tt.tt_ctx_set_option(ctx, "split", False)
+    S0, G0 = tt.tt_semblance_grad(ctx, th)
+    ctx.close()
+    assert (S - S0).abs().max().item() <= 1e-6
+    scale = G0.abs().flatten(0, 1).median(0).values
+    assert ((G - G0).abs() <= 1e-3 * (G0.abs() + scale)).all()
+
+
 def _cfg(op, np_, ng, **kw):
     kw = {"exch_every": 0, "polish_steps": 0, "polish_lr": 2e-4, "adapt": 0, **kw}
     lo, hi = BOUNDS[op]
