@@ -388,3 +388,38 @@ def test_stack_of_interleaved_groups(storage):
         outs.append(back)
     assert np.array_equal(outs[0], outs[1]) and np.array_equal(outs[0], outs[2])
     assert times[0] <= 1.4 * times[1], times
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+def test_forms_agree_on_infinities_and_nans(storage):
+    """Records with infinite and NaN samples: every form of a launch has the same
+    values and the same NaNs (evaluation by a warp a slice and a warp for eight;
+    fused and stepwise search; stack by lanes and by warps)."""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    n_dom, sizes = 8 * n_sm, (int(0.8 * n_sm),)
+    x, mid, off = _line(60, 300)
+    off[:4] = 5.0  # early windows read the samples below
+    x[0, 30:40], x[1, 90:100], x[2, 150:160] = np.inf, np.nan, -np.inf
+    prob = _problem(n_dom, sizes, 60, 300)
+    th = to_dev(random_theta(n_dom, 16, *BOUNDS[1], 7))
+
+    def same(a, b):
+        return torch.equal(a.isnan(), b.isnan()) and torch.equal(a.nan_to_num(), b.nan_to_num())
+
+    ctx = tt.tt_ctx_create(x, mid, off, prob, None, storage=storage, device=dev())
+    few, many = tt.tt_semblance_eval(ctx, th[:, :8].contiguous()), tt.tt_semblance_eval(ctx, th)
+    lanes = tt.tt_stack(ctx, th[:, 0].contiguous())
+    ctx.close()
+    own = _problem(n_dom, sizes, 60, 300, own_groups=True)
+    ctx = tt.tt_ctx_create(x, mid, off, own, None, storage=storage, device=dev())
+    warps = tt.tt_stack(ctx, th[:, 0].contiguous())
+    ctx.close()
+    assert few.isnan().any() and (few == 0).any() and same(few, many[:, :8])
+    assert lanes.isnan().any() and same(lanes, warps)
+    prob = _problem(2 * n_sm, (60,), 60, 300)
+    ctx = tt.tt_ctx_create(x, mid, off, prob, _cfg(1, 32, 4), storage=storage, device=dev())
+    th1, S1, _ = tt.tt_search(ctx)
+    tt.tt_ctx_profile(ctx, True)
+    th2, S2, _ = tt.tt_search(ctx)
+    ctx.close()
+    assert torch.equal(th1, th2) and same(S1, S2)
