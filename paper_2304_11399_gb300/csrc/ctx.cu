@@ -69,6 +69,41 @@ tt::EvalArgs tt_ctx::eval_args(const float* theta, int P, float* S) const {
   return a;
 }
 
+static void use_scratch(tt::EvalArgs& a, const tt::SplitScratch& s) {
+  a.part = s.part;
+  a.part_Ed = s.part_Ed;
+  a.ticket = s.ticket;
+}
+
+tt::EvalArgs tt_ctx::search_args(const float* theta, int P, float* S) const {
+  tt::EvalArgs a = eval_args(theta, P, S);
+  use_scratch(a, split_search);
+  return a;
+}
+
+// Evaluations of one context may overlap on different streams, so that only the
+// stream that came first has the scratch; a captured launch, which a graph may
+// replay on any stream, has none.
+tt::EvalArgs tt_ctx::call_args(const float* theta, int P, float* S, cudaStream_t s) {
+  tt::EvalArgs a = eval_args(theta, P, S);
+  if (!split_eval.part) return a;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  cudaError_t e = cudaStreamIsCapturing(s, &st);
+  if (e == cudaSuccess && st != cudaStreamCaptureStatusNone) return a;
+  if (e == cudaSuccess) e = cudaStreamGetId(s, &id);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return a;
+  }
+  if (!split_owned) {
+    split_owned = true;
+    split_stream = id;
+  }
+  if (split_stream == id) use_scratch(a, split_eval);
+  return a;
+}
+
 void tt_ctx_drop_graph(tt_ctx* c) {
   if (c->graph_exec) {
     cudaGraphExecDestroy(c->graph_exec);
@@ -356,6 +391,9 @@ void free_ctx(tt_ctx* c) {
                   c->trial[1], c->tfit[0], c->tfit[1], c->snap, c->imports, c->slots,
                   c->best_idx, c->pol_th, c->pol_g, c->pol_S, c->pol_bth, c->pol_bS, c->d_err,
                   c->queue, c->probe, c->out_th,
+                  c->split_eval.part, c->split_eval.part_Ed, c->split_eval.ticket,
+                  c->split_search.part, c->split_search.part_Ed, c->split_search.ticket,
+                  c->split_side.part, c->split_side.part_Ed, c->split_side.ticket,
                   c->out_S, c->jade_mu, c->jade_arc, c->jade_F,
                   c->jade_CR, c->jade_na};
   for (void* p : ptrs)
@@ -625,6 +663,17 @@ extern "C" tt_status tt_ctx_create(tt_ctx** out, const tt_gathers* ga, const tt_
   }
   TRY(dalloc(&c->queue, 2), "alloc queue");
   TRY(dalloc(&c->probe, tt::kProbeFloats), "alloc probe window");
+  if (c->n_dom > 0 && c->sum_N >= double(tt::kSplitScratchMinAp) * c->n_dom) {
+    for (tt::SplitScratch* p : {&c->split_eval, &c->split_search, &c->split_side}) {
+      if (p != &c->split_eval && !c->has_cfg) continue;  // no search without settings
+      const size_t sets = size_t(tt::split_sets(c->n_sm)) * 64;
+      const size_t units = size_t(tt::split_tickets(c->n_sm));
+      TRY(dalloc(&p->part, sets * (2 * c->W + 2)), "alloc split scratch");
+      if (c->storage == TT_STORE_BF16) TRY(dalloc(&p->part_Ed, sets), "alloc split scratch");
+      TRY(dalloc(&p->ticket, units), "alloc split tickets");
+      TRY(cudaMemsetAsync(p->ticket, 0, units * sizeof(unsigned), s), "clear split tickets");
+    }
+  }
   {
     size_t nd = size_t(c->n_dom), Dz = size_t(D);
     TRY(dalloc(&c->out_th, nd * Dz), "alloc search output");

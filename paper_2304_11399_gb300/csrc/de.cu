@@ -299,7 +299,7 @@ extern "C" tt_status tt_neighbor_exchange(tt_ctx* c, int32_t n_m0, int32_t n_t0,
                                                             best_theta, pop, fit, imp, sl, s)),
                      "exchange launch");
   if (st != TT_OK) return st;
-  tt::EvalArgs a = c->eval_args(imp, 4, fit);
+  tt::EvalArgs a = c->search_args(imp, 4, fit);
   a.slots = sl;
   a.np_out = c->cfg.np;
   return tt_cuda_check(c, c->semblance(a, s, false), "import evaluation");

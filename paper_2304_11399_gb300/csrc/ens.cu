@@ -216,8 +216,9 @@ tt_status ens_body(tt_ctx* c, const tt_ens_cfg& e, float* bth, float* bS, cudaSt
   // The interpolated samples of a step (interpolate, evaluate, keep) only
   // touch that trace's skipped samples, which the next steps of the stage do
   // not read; they run on the side stream, overlapping the next step, with
-  // their maps and buffers double-buffered by step parity and a work counter of
-  // their own (a persistent launch clears its counter and takes units from it).
+  // their maps and buffers double-buffered by step parity and a work counter and
+  // split scratch of their own (a persistent launch clears its counter and takes
+  // units from it).
   // A step waits for the side work of the step two before it (which used the
   // same buffers); every stage ends with a join.
   if (!c->side_stream) {
@@ -275,7 +276,7 @@ tt_status ens_body(tt_ctx* c, const tt_ens_cfg& e, float* bth, float* bS, cudaSt
             gen0, c->bounds, c->bounds + D, c->cfg.adapt ? c->jade_mu : nullptr, c->jade_na,
             c->cfg.F, c->cfg.CR);
         STEP(c->counted(cudaGetLastError()), "ens init");
-        tt::EvalArgs ea = c->eval_args(c->pop, NP, c->fit);
+        tt::EvalArgs ea = c->search_args(c->pop, NP, c->fit);
         ea.n_dom = n_est_loc;
         ea.dom_map = map_est;
         if (sg.bf) {  // the own best's semblance is known: NP - 1 pairs per sample
@@ -299,7 +300,7 @@ tt_status ens_body(tt_ctx* c, const tt_ens_cfg& e, float* bth, float* bS, cudaSt
           a.tfit = pending ? c->tfit[cur ^ 1] : nullptr;
           a.next = c->trial[cur];
           STEP(c->counted(tt::launch_de_step(a, s)), "ens de step");
-          tt::EvalArgs et = c->eval_args(c->trial[cur], NP, c->tfit[cur]);
+          tt::EvalArgs et = c->search_args(c->trial[cur], NP, c->tfit[cur]);
           et.n_dom = n_est_loc;
           et.dom_map = map_est;
           STEP(c->semblance(et, s, false), "ens evaluate trial");
@@ -331,10 +332,13 @@ tt_status ens_body(tt_ctx* c, const tt_ens_cfg& e, float* bth, float* bS, cudaSt
         STEP(cudaStreamWaitEvent(s2, fork_ev[par], 0), "ens fork");
         k_ens_interp<<<blocks(n_skp_loc), 256, 0, s2>>>(g, D, map_skp, bth, th_skp);
         STEP(c->counted(cudaGetLastError()), "ens interpolate");
-        tt::EvalArgs ei = c->eval_args(th_skp, 1, S_skp);
+        tt::EvalArgs ei = c->search_args(th_skp, 1, S_skp);
         ei.n_dom = n_skp_loc;
         ei.dom_map = map_skp;
         ei.queue = c->queue + 1;
+        ei.part = c->split_side.part;
+        ei.part_Ed = c->split_side.part_Ed;
+        ei.ticket = c->split_side.ticket;
         STEP(c->semblance(ei, s2, false), "ens evaluate interpolated");
         calls += (unsigned long long)active * g.n_skp;
         k_ens_keep<<<blocks(n_skp_loc), 256, 0, s2>>>(n_skp_loc, D, map_skp, th_skp, S_skp, bth,

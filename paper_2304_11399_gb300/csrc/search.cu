@@ -24,7 +24,7 @@ tt_status polish_impl(tt_ctx* c, const float* theta_in, float* theta_out, float*
       "polish copy");
   if (st != TT_OK) return st;
   for (int k = 0; k < steps; ++k) {
-    tt::EvalArgs a = c->eval_args(c->pol_th, 1, c->pol_S);
+    tt::EvalArgs a = c->search_args(c->pol_th, 1, c->pol_S);
     a.dS = c->pol_g;
     // The iterates' S are compared: unsplit, so that their sums are of one order
     // whatever the number of domains. The last iterate's S, below, is a plain
@@ -39,7 +39,7 @@ tt_status polish_impl(tt_ctx* c, const float* theta_in, float* theta_out, float*
                        "polish update");
     if (st != TT_OK) return st;
   }
-  tt::EvalArgs a = c->eval_args(c->pol_th, 1, c->pol_S);
+  tt::EvalArgs a = c->search_args(c->pol_th, 1, c->pol_S);
   st = tt_cuda_check(c, c->semblance(a, s, false), "polish evaluation");
   if (st != TT_OK) return st;
   st = tt_cuda_check(c, c->counted(tt::launch_polish_update(n, D, c->pol_th, c->pol_g,
@@ -107,14 +107,14 @@ tt_status search_body(tt_ctx* c, float* best_theta, float* best_S, cudaStream_t 
   const bool order = (c->member_order == 1 || (c->member_order == 2 && long_apertures)) &&
                      NP > 1 && NP <= tt::kOrderMaxP;
   auto evaluate = [&](const float* th, float* fit, float* tmp, float* tmp_fit) -> tt_status {
-    if (!order) return tt_cuda_check(c, c->semblance(c->eval_args(th, NP, fit), s, false),
+    if (!order) return tt_cuda_check(c, c->semblance(c->search_args(th, NP, fit), s, false),
                                      "evaluate");
     int* map = reinterpret_cast<int*>(tmp_fit);
     tt_status r = tt_cuda_check(
-        c, c->counted(tt::launch_member_order(c->eval_args(th, NP, nullptr), tmp, map, s)),
+        c, c->counted(tt::launch_member_order(c->search_args(th, NP, nullptr), tmp, map, s)),
         "member order");
     if (r != TT_OK) return r;
-    tt::EvalArgs ea = c->eval_args(tmp, NP, fit);
+    tt::EvalArgs ea = c->search_args(tmp, NP, fit);
     ea.slots = map;
     ea.np_out = NP;
     return tt_cuda_check(c, c->semblance(ea, s, false), "evaluate");
@@ -140,13 +140,13 @@ tt_status search_body(tt_ctx* c, float* best_theta, float* best_S, cudaStream_t 
                                              prev ? slab->recv_prev : nullptr,
                                              next ? slab->recv_next : nullptr)),
          "exchange");
-    tt::EvalArgs ea = c->eval_args(c->imports, 4, c->fit);
+    tt::EvalArgs ea = c->search_args(c->imports, 4, c->fit);
     ea.slots = c->slots;
     ea.np_out = NP;
     STEP(c->semblance(ea, s, false), "evaluate imports");
     return TT_OK;
   };
-  tt::EvalArgs whole = c->eval_args(c->pop, NP, c->fit);
+  tt::EvalArgs whole = c->search_args(c->pop, NP, c->fit);
   if (!c->profiling && c->member_order != 1 && tt::fused_search_fits(whole)) {
     // all generations up to the next exchange in one launch
     for (int g = 0; g <= NG;) {

@@ -3,6 +3,8 @@
 // split forms), the adjoint gradient (K2) and the stacked output.
 #include "semblance_kernels.cuh"
 
+#include <cmath>
+
 namespace tt {
 namespace sk {
 extern template KFn pick_kernel<TT_OP_CMP>(int, int, int, bool);
@@ -52,6 +54,24 @@ int split_blocks(long long units, int n_sm) {
                                                        : 1;
 }
 
+// Whether a launch of B blocks a unit adds its blocks' sums through the scratch (if
+// it has one) rather than in clusters. A launch takes as long as the SM with the most
+// blocks, and clusters, placed whole within a part of the chip, do not fill every
+// SM: 61 of nine blocks and 83 of seven fit at four blocks an SM (occupancy query)
+// where 67 and 86 times as many single blocks do, 0.905 and (over all numbers of
+// blocks an SM) 0.93 of them. Where that is one block more for some SM, single blocks
+// win (FP32, w = 5, 5000 traces, 48 / 62 / 125 / 149 / 167 / 299 units 52 / 65 / 112 /
+// 128 / 143 / 237 us against 62 / 75 / 125 / 147 / 154 / 250; BF16, w = 8, 62 / 149
+// units 104 / 208 us against 121 / 244); elsewhere the way through global memory costs
+// 2 to 5 us more (36 / 77 / 119 / 179 units 52 / 79 / 112 / 157 against 51 / 77 / 109 /
+// 157), which apertures below 1500 traces do not win back either way (1008 traces,
+// 118 / 152 / 282 units 34 / 41 / 64 against 32 / 40 / 61).
+bool scratch_wins(const EvalArgs& a, long long units, int B) {
+  if (B < kSplitSmallBlocks || a.mean_ap < kSplitScratchMinAp) return false;
+  const double per_sm = double(units * B) / a.n_sm;
+  return std::ceil(per_sm / (B == kSplitTinyBlocks ? 0.905 : 0.93)) > std::ceil(per_sm);
+}
+
 cudaError_t launch_split(EvalArgs& a, long long units, bool mv, cudaStream_t s) {
   const bool bf = a.storage == TT_STORE_BF16;
   const int B = split_blocks(units, a.n_sm);
@@ -72,6 +92,12 @@ cudaError_t launch_split(EvalArgs& a, long long units, bool mv, cudaStream_t s) 
     const cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return e;
     fn<<<unsigned(units), 32 * kSplitSmallBlocks, smem, s>>>(a);
+    return cudaGetLastError();
+  }
+  if (a.part && scratch_wins(a, units, B)) {  // a block's own eight sets fit without asking
+    const KFn fn = pick(sk::kKindSplitGlobal, a, mv);
+    if (!fn) return cudaErrorInvalidValue;
+    fn<<<unsigned(units * B), 32 * sk::kSplitWarps, sk::split_smem_bytes(1, a.W, bf), s>>>(a);
     return cudaGetLastError();
   }
   const KFn fn = pick(sk::kKindSplit, a, mv);
@@ -359,9 +385,9 @@ extern "C" tt_status tt_semblance_eval(tt_ctx* ctx, const float* theta, int32_t 
   if (!ctx) return tt_fail(nullptr, TT_ERR_INVALID_ARG, "ctx is NULL");
   if (P < 1) return tt_fail(ctx, TT_ERR_INVALID_ARG, "P must be >= 1");
   if (ctx->n_dom > 0 && (!theta || !S)) return tt_fail(ctx, TT_ERR_INVALID_ARG, "NULL array");
-  tt::EvalArgs a = ctx->eval_args(theta, P, S);
-  return tt_cuda_check(ctx, ctx->semblance(a, static_cast<cudaStream_t>(stream), false),
-                       "semblance launch");
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const tt::EvalArgs a = ctx->call_args(theta, P, S, s);
+  return tt_cuda_check(ctx, ctx->semblance(a, s, false), "semblance launch");
 }
 
 extern "C" tt_status tt_stack(tt_ctx* ctx, const float* theta, float* out, void* stream) {
@@ -409,12 +435,12 @@ extern "C" tt_status tt_semblance_eval_sums(tt_ctx* ctx, const float* theta, int
   if (!ctx) return tt_fail(nullptr, TT_ERR_INVALID_ARG, "ctx is NULL");
   if (P < 1) return tt_fail(ctx, TT_ERR_INVALID_ARG, "P must be >= 1");
   if (!theta || !S || !sums) return tt_fail(ctx, TT_ERR_INVALID_ARG, "NULL array");
-  tt::EvalArgs a = ctx->eval_args(theta, P, S);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  tt::EvalArgs a = ctx->call_args(theta, P, S, s);
   if (tt::grad_sums_bytes(a) <= 0)
     return tt_fail(ctx, TT_ERR_INVALID_ARG, "this launch keeps no sums");
   set_sums(a, sums);
-  return tt_cuda_check(ctx, ctx->semblance(a, static_cast<cudaStream_t>(stream), false),
-                       "semblance launch");
+  return tt_cuda_check(ctx, ctx->semblance(a, s, false), "semblance launch");
 }
 
 extern "C" tt_status tt_semblance_grad_sums(tt_ctx* ctx, const float* theta, int32_t P,

@@ -446,7 +446,7 @@ __device__ __forceinline__ void eval_unit(const EvalArgs& a, long long unit, int
 // every variant of a launch gives the same bits -- and results stay
 // reproducible. Three kernels run it, with the same bits:
 //  * k_semblance_split: a warp per slice, eight warps per block, a cluster of
-//    B blocks per unit. The blocks push their sums into the first one's shared
+//    B blocks per unit (or, for long apertures at some sizes, B single blocks). The blocks push their sums into the first one's shared
 //    memory and leave; no global scratch, fence, ticket or re-read. Latency
 //    bound (44% issue, 43% of the warps resident): a CRS launch of 118 units x
 //    1008 traces, w = 5, takes 30.9 us against 37.5 us through global scratch,
@@ -493,6 +493,8 @@ template <typename T>
 constexpr size_t split_smem_bytes_of(int B, int W) {
   return split_set_bytes<T>(W) * size_t(kSplitWarps + (B > 1 && !split_pulls<T>(W) ? B : 0));
 }
+static_assert(split_smem_bytes_of<__nv_bfloat16>(1, TT_MAX_HALF_WINDOW) + 512 <= 48 * 1024,
+              "a block's own sets fit without an opt-in");
 inline size_t split_smem_bytes(int B, int W, bool bf16) {
   return bf16 ? split_smem_bytes_of<__nv_bfloat16>(B, W) : split_smem_bytes_of<float>(B, W);
 }
@@ -521,7 +523,9 @@ __device__ __forceinline__ void finish_pair(const EvalArgs& a, long long q, int 
   store_S(a, q, a.slots ? dom_of(q, a.P) : 0, normalise<T>(Q, N, tot[K * 64], Ed));
 }
 
-template <int OP, int W, typename T, bool MV>
+// GLOBAL: no clusters; the blocks' sums meet in the launch's scratch, where the
+// unit's last block to arrive adds them (launch_split says when).
+template <int OP, int W, typename T, bool MV, bool GLOBAL>
 __global__ void __launch_bounds__(32 * kSplitWarps, 4) k_semblance_split(const EvalArgs a) {
   constexpr int K = 2 * W + 1, R = K + 1;
   constexpr int S = kSplitWarps, NT = 32 * S;
@@ -535,11 +539,11 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 4) k_semblance_split(const E
   const int rank = int(blockIdx.x - unit * B);
   double* part_Ed = reinterpret_cast<double*>(split_smem);  // [S][64], then [B][64]
   double* recv_Ed = part_Ed + S * 64;
-  const int sets = S + (B > 1 && !PULL ? B : 0);
+  const int sets = S + (B > 1 && !PULL && !GLOBAL ? B : 0);
   float* part = reinterpret_cast<float*>(part_Ed + (Chunk<T>::kF64 ? sets * 64 : 0));
   float* recv = part + S * R * 64;  // [B][R][64], in the cluster's first block
   // met by cluster_wait below: every block has started
-  if (B > 1 && !PULL) cluster_arrive_relaxed();
+  if (B > 1 && !PULL && !GLOBAL) cluster_arrive_relaxed();
   const long long q0 = unit * 64 + lane, q1 = q0 + 32;
   Lane L0, L1;
   const bool v0 = lane_setup<OP, true>(a, q0, L0);
@@ -586,10 +590,13 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 4) k_semblance_split(const E
     }
   }
   __syncthreads();
-  // the block's sums, slices in order: to the cluster's first block
+  // the block's sums, slices in order: to the cluster's first block, or the scratch
   float* to = part;
   double* to_d = part_Ed;
-  if (B > 1 && !PULL) {
+  if constexpr (GLOBAL) {
+    to = a.part + blockIdx.x * size_t(R * 64);
+    to_d = a.part_Ed + blockIdx.x * size_t(64);
+  } else if (B > 1 && !PULL) {
     cluster_wait();
     to = cl.map_shared_rank(recv, 0) + rank * R * 64;
     to_d = cl.map_shared_rank(recv_Ed, 0) + rank * 64;
@@ -606,7 +613,24 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 4) k_semblance_split(const E
     to_d[threadIdx.x] = t;
   }
   double Ed = 0.0;
-  if (B > 1 && !PULL) {
+  if constexpr (GLOBAL) {  // no block waits
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(a.ticket + unit, 1u) == unsigned(B - 1);
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (threadIdx.x == 0) a.ticket[unit] = 0u;  // ready for the next launch
+    const size_t set0 = size_t(unit) * B;
+    for (int i = threadIdx.x; i < R * 64; i += NT) {
+      float t = 0.f;
+      for (int b = 0; b < B; ++b) t = __fadd_rn(t, __ldcg(a.part + (set0 + b) * (R * 64) + i));
+      part[i] = t;
+    }
+    if (Chunk<T>::kF64 && threadIdx.x < 64)
+      for (int b = 0; b < B; ++b) Ed += __ldcg(a.part_Ed + (set0 + b) * 64 + threadIdx.x);
+  } else if (B > 1 && !PULL) {
     __syncwarp();
     cluster_arrive();
     if (rank) return;  // done with: nothing of this block's shared memory is read by others
@@ -634,7 +658,7 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 4) k_semblance_split(const E
   }
   __syncthreads();
   if (threadIdx.x < 64) {
-    if (Chunk<T>::kF64 && B == 1) Ed = part_Ed[threadIdx.x];
+    if (Chunk<T>::kF64 && !GLOBAL && B == 1) Ed = part_Ed[threadIdx.x];
     finish_pair<W, T>(a, unit * 64 + threadIdx.x, size[threadIdx.x], part + threadIdx.x, Ed);
   }
 }
@@ -1539,7 +1563,7 @@ OFn pick_order(bool mv) {
 using SFn = void (*)(const EvalArgs, float*);
 enum KernelKind {
   kKindPacked = 0, kKindScalar = 1, kKindSplit = 2, kKindGrad = 3, kKindGradSplit = 4,
-  kKindGradAhead = 5, kKindShort = 6
+  kKindGradAhead = 5, kKindShort = 6, kKindSplitGlobal = 7
 };
 
 template <int OP, int W, typename T, bool MV>
@@ -1547,7 +1571,8 @@ KFn pick_kind(int kind) {
   switch (kind) {
     case kKindPacked: return k_semblance<OP, W, T, MV>;
     case kKindScalar: return k_semblance_scalar<OP, W, T, MV>;
-    case kKindSplit: return k_semblance_split<OP, W, T, MV>;
+    case kKindSplit: return k_semblance_split<OP, W, T, MV, false>;
+    case kKindSplitGlobal: return k_semblance_split<OP, W, T, MV, true>;
     case kKindShort: return k_semblance_short<OP, W, T, MV>;
     case kKindGrad: return k_semblance_grad<OP, W, T, MV, 1>;
     case kKindGradAhead: return k_semblance_grad<OP, W, T, MV, 6>;

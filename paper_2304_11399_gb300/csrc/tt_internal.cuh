@@ -27,6 +27,23 @@ constexpr int kSplitMultiPerSm = 12;
 constexpr int kSplitSmallBlocks = 7;
 constexpr int kSplitTinyBlocks = 9;
 
+// Global scratch of split launches with long apertures (see launch_split): B
+// sets of sums per unit and a count of its finished blocks, zero between
+// launches. Launches that share one must not overlap.
+struct SplitScratch {
+  float* part = nullptr;       // [split_sets][2 W + 2][64]
+  double* part_Ed = nullptr;   // BF16 storage: [split_sets][64]
+  unsigned* ticket = nullptr;  // [split_tickets]
+};
+// the most sets (units times blocks) and units of a launch of 7 or 9 blocks a unit
+inline long long split_sets(int n_sm) {
+  const long long small = (long long)n_sm * kSplitSmallPerSm * kSplitSmallBlocks;
+  const long long tiny = (long long)(n_sm / 2) * kSplitTinyBlocks;
+  return small > tiny ? small : tiny;
+}
+inline long long split_tickets(int n_sm) { return (long long)n_sm * kSplitSmallPerSm; }
+constexpr float kSplitScratchMinAp = 1500.f;  // mean aperture from which it is used
+
 // Padded trace layout: sample n of trace r lives at r * pitch + kPadFront + n.
 // kPadFront >= max half window; kPadBack >= 2 * max half window + 2 so that a
 // window whose position is clamped to ns + w reads only padding zeros.
@@ -61,6 +78,10 @@ struct EvalArgs {
   int block;                // threads per block: 128 or 256
   int split;                // 1: small forward launches split the aperture over warps
   int split_blocks;         // B of a split launch (set by the launcher)
+  // scratch of a multi-block split launch (see SplitScratch); NULL: clusters only
+  float* part;
+  double* part_Ed;
+  unsigned* ticket;
   int n_sm;                 // SMs of the device (split thresholds, persistent grid)
   unsigned long long* queue;  // persistent mode: work-unit counter, zero at launch
   // sums of a split launch, 64 pairs at a time: s_k and E [units][2 W + 2][64], BF16
@@ -233,6 +254,13 @@ struct tt_ctx {
   // persistent-kernel work counters: one of the calls, one of the launches that
   // the ENS sweep runs beside them on its side stream (each launch clears its own)
   unsigned long long* queue = nullptr;
+  // scratch of split launches with long apertures: of tt_semblance_eval, which
+  // uses it on one stream alone (`split_stream`, the first it was called on;
+  // stream ids are never reused), of the searches and of the ENS sweep's side
+  // stream
+  tt::SplitScratch split_eval, split_search, split_side;
+  bool split_owned = false;
+  unsigned long long split_stream = 0;
   float* probe = nullptr;   // window and sink of the L1 probe (kProbeFloats)
   // a side stream: the ENS sweep evaluates each step's interpolated samples
   // concurrently with the next step
@@ -270,6 +298,10 @@ struct tt_ctx {
   size_t ev_used = 0;
 
   tt::EvalArgs eval_args(const float* theta, int P, float* S) const;
+  // the same inside a search or a polish, whose calls must not overlap
+  tt::EvalArgs search_args(const float* theta, int P, float* S) const;
+  // and for a call's own evaluation on stream s
+  tt::EvalArgs call_args(const float* theta, int P, float* S, cudaStream_t s);
   // every semblance / gradient launch of the library goes through here
   cudaError_t semblance(const tt::EvalArgs& a, cudaStream_t s, bool grad);
   // a fused search launch, counted as the evaluations it holds

@@ -423,3 +423,77 @@ def test_forms_agree_on_infinities_and_nans(storage):
     th2, S2, _ = tt.tt_search(ctx)
     ctx.close()
     assert torch.equal(th1, th2) and same(S1, S2)
+
+
+@pytest.mark.parametrize("storage,w,P", [("f32", 5, 8), ("bf16", 8, 8), ("f32", 0, 2),
+                                         ("bf16", 3, 20)])
+def test_long_split_launches_on_several_streams(storage, w, P):
+    """Long apertures at unit counts (0.83, 0.41 and 0.96, 0.98 of a multiple of the
+    SMs' blocks) where the blocks' sums meet in the context's scratch: the stream
+    that evaluates first has it, another stream takes clusters, as a captured launch
+    does. The same bits in all three, and with both streams at work at once."""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    n_dom = {8: int(7.8 * n_sm), 2: int(13.2 * n_sm), 20: int(6.3 * n_sm)}[P]
+    x, mid, off = _line(200, 300)
+    prob = _problem(n_dom, (2000, 1500, 1700), 200, 300, w=w)
+    ctx = tt.tt_ctx_create(x, mid, off, prob, None, storage=storage, device=dev())
+    th = to_dev(random_theta(n_dom, P, *BOUNDS[1], 7))
+    S = tt.tt_semblance_eval(ctx, th)  # the first stream: with scratch
+    torch.cuda.synchronize()
+    other = torch.cuda.Stream(device=dev())
+    outs = [(torch.empty_like(S), torch.empty_like(S)) for _ in range(20)]
+    for a, b in outs:  # nothing between the streams
+        tt.tt_semblance_eval(ctx, th, a)
+        tt.tt_semblance_eval(ctx, th, b, stream=other)
+    torch.cuda.synchronize()
+    for a, b in outs:
+        assert torch.equal(a, S) and torch.equal(b, S)
+    T = torch.empty_like(S)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        tt.tt_semblance_eval(ctx, th, T)
+    T.zero_()
+    graph.replay()
+    again = tt.tt_semblance_eval(ctx, th)
+    torch.cuda.synchronize()
+    ctx.close()
+    assert torch.equal(T, S) and torch.equal(again, S)
+    if storage == "f32":
+        few = np.arange(0, n_dom, 97)
+        sub = dataclasses.replace(prob, dom_it0=prob.dom_it0[few], dom_group=prob.dom_group[few])
+        ref = oracle.semblance.semblance_many(x, mid, off, sub, th[few].cpu().numpy())
+        assert np.max(np.abs(S[few].cpu().numpy() - ref)) <= 1e-5
+
+
+def test_search_and_sweep_over_long_apertures():
+    """The search's and the ENS sweep's split launches over long apertures, whose
+    sums meet in scratch of their own: eager and replayed runs agree, beside
+    evaluations on another stream, and the semblance reported is the evaluation's."""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    n_m0, n_t0 = 4, 5 * n_sm // 4
+    n_dom = n_m0 * n_t0
+    x, mid, off = _line(200, 300)
+    prob = _problem(n_dom, (1600,) * n_m0, 200, 300)
+    prob.dom_group = np.repeat(np.arange(n_m0), n_t0).astype(np.int32)
+    prob.dom_it0 = np.tile(np.arange(n_t0), n_m0).astype(np.int32)
+    prob.n_m0, prob.n_t0 = n_m0, n_t0
+    ctx = tt.tt_ctx_create(x, mid, off, prob, _cfg(1, 12, 5, exch_every=2, polish_steps=2),
+                           device=dev())
+    th = to_dev(random_theta(n_dom, 12, *BOUNDS[1], 7))
+    S = tt.tt_semblance_eval(ctx, th)
+    other = torch.cuda.Stream(device=dev())
+    runs = []
+    for graph in (True, False):
+        tt.tt_ctx_set_option(ctx, "search_graph", graph)
+        for call in (lambda: tt.tt_search(ctx, stream=other),
+                     lambda: tt.tt_ens_search(ctx, 12, 2, 12, 2, 2, 1, 2, stream=other)):
+            best, bS, n = call()
+            for _ in range(4):
+                assert torch.equal(tt.tt_semblance_eval(ctx, th), S)
+            torch.cuda.synchronize()
+            E = tt.tt_semblance_eval(ctx, best[:, None].contiguous())[:, 0]
+            assert (E - bS).abs().max().item() <= 1e-5
+            runs.append((best, bS, n))
+    ctx.close()
+    for a, b in zip(runs[:2], runs[2:]):
+        assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1]) and a[2] == b[2]
