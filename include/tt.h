@@ -184,8 +184,8 @@ tt_status tt_semblance_grad(tt_ctx* ctx, const float* theta, int32_t P, float* S
  *       aligned), later tt_semblance_grad_sums with the same theta and P on the
  *       same traces: the gradient's second pass alone;
  *  0    tt_semblance_eval, later tt_semblance_grad;
- *  -1   tt_semblance_grad at once (a launch too small for the second pass to
- *       show beside its issue); its S is tt_semblance_eval's bit for bit.
+ *  -1   tt_semblance_grad at once (a launch whose two passes take less than
+ *       issuing them apart); its S is tt_semblance_eval's bit for bit.
  * TT_ERR_INVALID_ARG for NULL arrays, and from tt_semblance_eval_sums where
  * *bytes is not positive. */
 tt_status tt_semblance_sums_size(tt_ctx* ctx, int32_t P, int64_t* bytes);

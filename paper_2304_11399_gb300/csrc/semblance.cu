@@ -137,10 +137,13 @@ bool grad_split(const EvalArgs& a, long long units) {
          (a.mean_ap >= 256.f || (a.mean_ap >= 16.f && units < 16ll * a.n_sm));
 }
 
-// Pairs times aperture entries up to which a differentiated evaluation takes the
-// adjoint at once: there it runs 20 to 45 us, the evaluation 20, and a call takes
-// 33 us to issue (4 million: 52 to 59 us).
-constexpr double kGradTogetherMax = 2097152.0;
+// Pairs times aperture entries (half as many in BF16 storage, whose S is evaluated
+// as well) up to which a differentiated evaluation takes the adjoint at once. Both
+// ways a pass forward and backward is host time there, and the backward's own launch
+// adds 40 to 60 us of it (4,000 x 1008: 220 against 279 us); a value whose backward
+// never comes takes the adjoint's time instead of the evaluation's, at most some 80
+// us more (4,000 x 1008: 52 against 33 us; 16 million: about 140 against 60).
+constexpr double kGradTogetherMax = 16777216.0;
 
 // The cluster has the forward launch's B blocks, 9, 7, 2 or 1, so that S agrees
 // with it (1008 traces, clusters of 1 / 2 / 4 / 7 / 8 / 9: 24 units 107 / 61 / 36 /
@@ -261,16 +264,16 @@ cudaError_t launch_semblance_grad(const EvalArgs& a, cudaStream_t s) { return la
 // them (60,000 domains x 1008 traces: the value 197 us, with its gradient 483 us
 // through autograd, against 459 and 478 us with the adjoint at once and 197 and
 // 675 us with a launch of each; 300,000 x 144: 129 and 336 us, 307 and 325 us, 129
-// and 460 us). Where both passes are no longer than a call takes to issue, the
-// adjoint gives value and gradient at once (2,000 x 1008: 34 and 221 us against 38
-// and 301 us, which is host time). What the evaluation does not split, or holds
+// and 460 us). Where a pass is host time either way, the adjoint gives value and
+// gradient at once (kGradTogetherMax). What the evaluation does not split, or holds
 // apertures too short for split gradients, is evaluated and differentiated by
 // launches of their own.
 long long grad_sums_bytes(const EvalArgs& a) {
   const long long n = (long long)a.n_dom * a.P, units = (n + 63) / 64;
   if (!a.split || n == 0 || units >= (long long)a.n_sm * kSplitUnitsPerSm || a.mean_ap < 16.f)
     return 0;
-  if (double(n) * a.mean_ap <= kGradTogetherMax && grad_split(a, units)) return -1;
+  const double work = double(n) * a.mean_ap * (a.storage == TT_STORE_BF16 ? 2.0 : 1.0);
+  if (work <= kGradTogetherMax && grad_split(a, units)) return -1;
   return units * (long long)(a.storage == TT_STORE_BF16 ? sk::split_set_bytes<__nv_bfloat16>(a.W)
                                                         : sk::split_set_bytes<float>(a.W));
 }

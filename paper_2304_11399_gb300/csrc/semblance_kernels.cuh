@@ -446,9 +446,10 @@ __device__ __forceinline__ void eval_unit(const EvalArgs& a, long long unit, int
 // every variant of a launch gives the same bits -- and results stay
 // reproducible. Three kernels run it, with the same bits:
 //  * k_semblance_split: a warp per slice, eight warps per block, a cluster of
-//    B blocks per unit (or, for long apertures at some sizes, B single blocks). The blocks push their sums into the first one's shared
-//    memory and leave; no global scratch, fence, ticket or re-read. Latency
-//    bound (44% issue, 43% of the warps resident): a CRS launch of 118 units x
+//    B blocks per unit (for long apertures, at some sizes, B single blocks whose
+//    sums meet in global scratch: scratch_wins). A cluster's blocks push their
+//    sums into the first one's shared memory and leave; no fence, ticket or
+//    re-read. Latency bound (44% issue, 43% of the warps resident): a CRS launch of 118 units x
 //    1008 traces, w = 5, takes 30.9 us against 37.5 us through global scratch,
 //    258 units 63.0 us against 70.9 us, 24 units of 48 traces 9.7 against 12.5.
 //  * k_semblance_short: a warp per eight slices, walked one after the other,

@@ -403,14 +403,16 @@ class SemblanceFn(torch.autograd.Function):
     (default: whether theta requires a gradient); without one the call is
     tt_semblance_eval. With one it runs as tt_semblance_sums_size says: the
     evaluation keeps each pair's sums (2w + 2 floats a pair, held until the graph
-    is freed) and the backward is the adjoint's second pass alone; a call whose
-    device time hides behind its issue runs the adjoint at once and keeps
-    dS/dtheta; any other is evaluated now and differentiated by the backward. So a
-    value whose backward never comes costs an evaluation (60,000 CRS domains x 1008
-    traces 197 us, with its backward 483 us; as a launch of each, 675 us). The
-    contiguous theta is saved as well: changing it in place before the backward is
-    an error (a copy made of a strided theta is not watched). A backward after
-    tt_ctx_load_traces is taken on the traces then loaded."""
+    is freed) and the backward is the adjoint's second pass alone (60,000 CRS
+    domains x 1008 traces: 197 us for the value, 483 us with its gradient; as a
+    launch of each 675 us). Up to 16 million pairs times aperture entries (8 in
+    BF16 storage) the call runs the adjoint at once and keeps dS/dtheta: a pass
+    forward and backward is host time there and 40 to 60 us shorter for it, a value
+    whose backward never comes up to 80 us longer than tt_semblance_eval, which
+    gives the same. Launches that do not split are evaluated now and differentiated
+    by the backward. The contiguous theta is saved as well: changing it in place
+    before the backward is an error (a copy made of a strided theta is not watched).
+    A backward after tt_ctx_load_traces is taken on the traces then loaded."""
 
     @staticmethod
     def forward(fctx, ctx: Context, theta: torch.Tensor, adjoint=None):

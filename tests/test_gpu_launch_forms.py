@@ -253,12 +253,13 @@ def test_gradient_of_infinite_energy(n_dom, P, sizes, op, w, ns, storage, bad):
 
 @pytest.mark.parametrize("n_dom,P,sizes,op,w,storage,ns,split,launches,same", [
     (60, 2, (48,), 1, 5, "f32", 300, True, 1, True),          # the adjoint at once
-    (4001, 1, (600, 590), 1, 5, "f32", 300, True, 2, True),   # sums of clusters of 9
-    (4001, 1, (600, 590), 2, 8, "bf16", 300, True, 2, True),
-    (19000, 1, (150, 140), 1, 5, "f32", 2200, True, 2, True),  # of slices walked by 7 warps
-    (6333, 3, (250, 0), 1, 3, "bf16", 300, True, 2, True),
-    (60001, 1, (48,), 1, 5, "f32", 300, True, 2, True),       # of clusters of 2
-    (170000, 1, (60, 17), 1, 5, "bf16", 300, True, 2, False),  # of one block; K2 does not split
+    (19000, 1, (150, 140), 1, 5, "f32", 2200, True, 1, True),
+    (4001, 1, (6000, 5900), 1, 5, "f32", 300, True, 2, True),  # sums, through scratch
+    (3800, 1, (3000, 2990), 2, 8, "bf16", 300, True, 2, True),  # of clusters of 9
+    (19456, 1, (900, 880), 1, 5, "f32", 2200, True, 2, True),  # of clusters of 7
+    (19000, 3, (370, 0), 1, 3, "bf16", 300, True, 2, True),   # of clusters of 2
+    (150001, 1, (130,), 1, 5, "f32", 300, True, 2, True),     # of one block
+    (170000, 1, (60, 60), 1, 5, "bf16", 300, True, 2, False),  # K2 does not split
     (117001, 1, (300,), 1, 1, "f32", 300, True, 2, True),
     (300000, 1, (8,), 1, 5, "f32", 300, True, 2, True),       # too short: two launches
     (312000, 1, (20,), 1, 5, "f32", 300, True, 2, True),      # too many pairs to split
